@@ -17,6 +17,7 @@
 #include "dmr_kernels.cuh"
 #include "dmr_adjoint.cuh"
 #include "dmr_period.cuh"
+#include "dmr_multi.cuh"
 
 namespace {
 
@@ -267,6 +268,8 @@ struct Base {
   bool in_batch = false;               // a run of a batch (its launches go through segment tables)
   cudaGraphExec_t gexec = nullptr;
   int g_cpar = 0, g_fpar = 0, g_rvalid = 0;   // state the graph was captured in
+  int g_cend = 0, g_fend = 0;                 // buffer parities its launches leave
+  bool strips = false;                 // one launch per EM (sub-)step only (set by an explicit launch shape)
   std::vector<int32_t> replay;
   size_t replay_pos = 0;
   bool has_fine = false;
@@ -1055,6 +1058,273 @@ struct Engine final : Base {
     return launched("EM step");
   }
 
+
+  // ---- several coarse steps per launch (dmr_multi.cuh) ---------------------
+  static constexpr int kMC = 2;       // node columns per lane of the tiles
+  static constexpr int kNearBlocks = 16;
+  static constexpr size_t kMaxSmem = 227 * 1024 - 1024;
+  // builds of the kernels: rows per warp, threads per block at most
+  struct TileKernel { int R, TH; void (*f)(dmr::MultiArgs<T>); };
+  struct NearKernel { int R, TH; void (*f)(dmr::MultiArgs<T>, dmr::NearArgs<T>); };
+  static std::vector<TileKernel> tile_kernels() {
+    if constexpr (sizeof(T) == 4)
+      return {{2, 1024, dmr::k_multi<T, kMC, 2, 1024>}, {4, 512, dmr::k_multi<T, kMC, 4, 512>}};
+    else return {};
+  }
+  static std::vector<NearKernel> near_kernels() {
+    if constexpr (sizeof(T) == 4) return {{1, 1024, dmr::k_near<T, 1, 1024>}, {2, 1024, dmr::k_near<T, 2, 1024>}};
+    else return {};
+  }
+  struct MultiPlan {
+    int K = 0;             // coarse steps per launch
+    bool ok = false;
+    int rect[4] = {-1, -1, -1, -1};
+    int zone[4], win[4];   // nodes (i0, j0, i1, j1) the near region stores / steps
+    int tk = -1, twarps = 0, tiles = 0, tw = 0, th = 0, gx = 0, gy = 0, hx = 0;   // tiles (tk < 0: none)
+    size_t tsmem = 0;
+    int nk = -1, nwarps = 0, crow = 0, frow = 0;                                   // near region (nk < 0: none)
+    size_t nsmem = 0;
+  };
+  std::vector<MultiPlan> mplans;
+  int multi_k = 0;         // coarse steps per launch (0: chosen by rule, 1: strips)
+  cudaStream_t st_near = nullptr;      // the near region runs beside the tiles
+  cudaEvent_t ev_fork = nullptr, ev_join = nullptr;
+
+  bool multi_allowed() const {
+    return sizeof(T) == 4 && !strips && multi_k != 1 && d.boundary == 0 && !timing && !in_batch && !persist_on();
+  }
+
+  // Launch shape for K coarse steps per launch from the present rectangle; not
+  // ok where a one-step launch is the better one or the kernels do not take
+  // the run: a mesh smaller than a tile, or a rectangle (with its coarse
+  // window) of more rows than the near region's warps hold at two rows each.
+  // (At eight rows per warp a 209 x 193 patch at r = 4 took 15.1 us per coarse
+  // step against 12.0 for the strips.)
+  MultiPlan multi_plan(int K) {
+    MultiPlan P;
+    P.K = K;
+    for (int q = 0; q < 4; ++q) P.rect[q] = has_fine ? rect[q] : -1;
+    const int r = cfg.r, nx = cfg.nx, ny = cfg.ny;
+    for (const auto& k : tile_kernels())
+      cudaFuncSetAttribute(k.f, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kMaxSmem);
+    for (const auto& k : near_kernels()) {
+      cudaFuncSetAttribute(k.f, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kMaxSmem);
+      cudaFuncSetAttribute(k.f, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+    }
+    P.zone[0] = P.zone[1] = 1; P.zone[2] = P.zone[3] = 0;
+    bool whole = false;           // the near region is the whole domain: no tiles
+    if (has_fine) {
+      auto fits = [&](int m) {
+        const int lo[2] = {std::max(rect[0] - m, 0), std::max(rect[1] - m, 0)};
+        const int hi[2] = {std::min(rect[2] + m, nx), std::min(rect[3] + m, ny)};
+        P.win[0] = lo[0]; P.win[1] = lo[1]; P.win[2] = hi[0]; P.win[3] = hi[1];
+        P.crow = std::max(2, (hi[1] - lo[1] + kNearBlocks - 1) / kNearBlocks);
+        P.frow = r * ((rect[3] - rect[1] + kNearBlocks - 1) / kNearBlocks);
+        const int fcols = r * (rect[2] - rect[0]) + 1, ccols = hi[0] - lo[0] + 1;
+        P.nsmem = dmr::near_smem<T>(ccols - 1, P.crow, fcols - 1, P.frow, r, rect[2] - rect[0], rect[3] - rect[1], K);
+        P.nk = -1;
+        if (P.nsmem > kMaxSmem) return false;
+        const auto kn = near_kernels();
+        for (size_t q = 0; q < kn.size() && P.nk < 0; ++q) {
+          P.nwarps = dmr::near_units(fcols, P.frow + 1, kn[q].R) + dmr::near_units(ccols, P.crow + 1, kn[q].R);
+          if (32 * P.nwarps > kn[q].TH) continue;
+          cudaLaunchConfig_t lc = {};
+          cudaLaunchAttribute la[2];
+          multi_config(&lc, la, kNearBlocks, P.nwarps, P.nsmem, kNearBlocks, false);
+          int n = 0;
+          if (cudaOccupancyMaxActiveClusters(&n, kn[q].f, &lc) == cudaSuccess && n > 0) P.nk = (int)q;
+          else cudaGetLastError();
+        }
+        return P.nk >= 0;
+      };
+      const int all = std::max(nx, ny);
+      if ((double)nx * ny <= kWholeCells && fits(all)) whole = true;
+      else if (!fits(2 * K + 1)) return P;
+      const int m = whole ? all : K;
+      P.zone[0] = std::max(rect[0] - m, 0); P.zone[1] = std::max(rect[1] - m, 0);
+      P.zone[2] = std::min(rect[2] + m, nx); P.zone[3] = std::min(rect[3] + m, ny);
+    }
+    if (whole) {
+      P.ok = true;
+      return P;
+    }
+    constexpr int W = 32 * kMC;
+    P.hx = (K + kMC - 1) / kMC * kMC;
+    P.tw = W - 2 * P.hx;
+    if (P.tw < 8 || nx + 1 < W) return P;
+    P.gx = (nx + 1 + P.tw - 1) / P.tw;
+    // the kernel and the rows per tile: the fewest rows that the busiest SM has to step
+    const int sms = std::max(1, num_sms - (has_fine ? kNearBlocks : 0));
+    double best = 1e300;
+    const auto kt = tile_kernels();
+    for (size_t q = 0; q < kt.size(); ++q)
+      for (int w = 4; w <= kt[q].TH / 32; ++w) {
+        const int H = w * kt[q].R, th = H - 2 * K;
+        if (th < 1 || H > ny + 1) continue;
+        const int tiles = P.gx * ((ny + 1 + th - 1) / th);
+        const double cost = (double)((tiles + sms - 1) / sms) * H;
+        if (cost >= best) continue;
+        best = cost;
+        P.tk = (int)q;
+        P.twarps = w;
+        P.th = th;
+        P.tiles = tiles;
+        P.gy = tiles / P.gx;
+        P.tsmem = dmr::tile_smem<T, kMC>(w, K);
+      }
+    P.ok = P.tk >= 0;
+    return P;
+  }
+  // a domain of at most this many cells is stepped whole by the near region's
+  // cluster, half a period per launch (96^2: 3.8 us per coarse step; tiles of
+  // a domain this small would be mostly halo)
+  static constexpr double kWholeCells = 20000.0;
+
+  // the plan for K steps, kept while the rectangle stays
+  const MultiPlan& multi_get(int K) {
+    for (auto it = mplans.begin(); it != mplans.end();) {
+      bool same = true;
+      for (int q = 0; q < 4; ++q) same = same && it->rect[q] == (has_fine ? rect[q] : -1);
+      if (!same) { it = mplans.erase(it); continue; }
+      if (it->K == K) return *it;
+      ++it;
+    }
+    mplans.push_back(multi_plan(K));
+    return mplans.back();
+  }
+  void multi_config(cudaLaunchConfig_t* lc, cudaLaunchAttribute* la, int grid, int warps, size_t smem, int ncl,
+                    bool pdl) const {
+    lc->gridDim = dim3((unsigned)grid);
+    lc->blockDim = dim3(32 * warps);
+    lc->dynamicSmemBytes = smem;
+    lc->stream = st;
+    int n = 0;
+    if (ncl) {
+      la[n].id = cudaLaunchAttributeClusterDimension;
+      la[n].val.clusterDim.x = (unsigned)ncl;
+      la[n].val.clusterDim.y = la[n].val.clusterDim.z = 1;
+      ++n;
+    }
+    if (pdl) {
+      la[n].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+      la[n].val.programmaticStreamSerializationAllowed = 1;
+      ++n;
+    }
+    lc->attrs = n ? la : nullptr;
+    lc->numAttrs = (unsigned)n;
+  }
+
+  // Launch P.K coarse steps from level mlev: coarse parity cp to cp ^ 1, fine
+  // parity fp to fd.  Tiles on the run's stream, the near region beside them
+  // on a stream of its own that starts and ends with them.
+  int go_multi(const MultiPlan& P, int64_t mlev, int cp, int fp, int fd, bool pdl) {
+    dmr::MultiArgs<T> A{};
+    auto mesh = [&](dmr::MultiMesh<T>* M, const dmr::Mesh<T>& m, int rr, int64_t level) {
+      M->m = m;
+      M->c = make_step(rr, level, true);
+      M->ps = ph[rr == 1 ? 0 : 2];
+      M->pc = ph[rr == 1 ? 1 : 3];
+      M->N = rr * cfg.steps_per_period;
+      M->q0 = (int)(level % M->N);
+    };
+    dmr::Mesh<T> src = C;
+    src.Ex = cE[cp][0]; src.Ey = cE[cp][1]; src.Hz = cE[cp][2]; src.vx = cE[cp][3]; src.vy = cE[cp][4];
+    mesh(&A.C, src, 1, mlev);
+    for (int q = 0; q < 5; ++q) A.C.d[q] = cE[cp ^ 1][q];
+    A.K = P.K;
+    A.hx = P.hx; A.tw = P.tw; A.th = P.th; A.gx = P.gx; A.gy = P.gy;
+    A.z0 = P.zone[0]; A.z1 = P.zone[1]; A.z2 = P.zone[2]; A.z3 = P.zone[3];
+    const bool both = P.nk >= 0 && P.tk >= 0;
+    if (both) {
+      if (!st_near) {
+        int lo = 0, hi = 0;
+        cudaDeviceGetStreamPriorityRange(&lo, &hi);
+        if (int s = ck(cudaStreamCreateWithPriority(&st_near, cudaStreamNonBlocking, hi), "near stream")) return s;
+        if (int s = ck(cudaEventCreateWithFlags(&ev_fork, cudaEventDisableTiming), "event")) return s;
+        if (int s = ck(cudaEventCreateWithFlags(&ev_join, cudaEventDisableTiming), "event")) return s;
+      }
+      if (int s = ck(cudaEventRecord(ev_fork, st), "fork")) return s;
+      if (int s = ck(cudaStreamWaitEvent(st_near, ev_fork, 0), "fork")) return s;
+    }
+    cudaLaunchAttribute la[2];
+    if (P.nk >= 0) {
+      dmr::NearArgs<T> N{};
+      mesh(&N.F, fine_at(fp), cfg.r, (int64_t)cfg.r * mlev);
+      for (int q = 0; q < 5; ++q) N.F.d[q] = fineE(cur, fd, q);
+      N.r = cfg.r;
+      N.restr = d.coupling == 0;
+      N.I0 = rect[0]; N.J0 = rect[1]; N.I1 = rect[2]; N.J1 = rect[3];
+      N.wi = P.win[0]; N.wj = P.win[1]; N.wnx = P.win[2] - P.win[0]; N.wny = P.win[3] - P.win[1];
+      N.cmode[dmr::SIDE_LEFT] = P.win[0] == 0 ? dmr::BC_MUR : dmr::BC_FROZEN;
+      N.cmode[dmr::SIDE_BOTTOM] = P.win[1] == 0 ? dmr::BC_MUR : dmr::BC_FROZEN;
+      N.cmode[dmr::SIDE_RIGHT] = P.win[2] == cfg.nx ? dmr::BC_MUR : dmr::BC_FROZEN;
+      N.cmode[dmr::SIDE_TOP] = P.win[3] == cfg.ny ? dmr::BC_MUR : dmr::BC_FROZEN;
+      for (int q = 0; q < 4; ++q) N.fmode[q] = side_on_edge(q) ? dmr::BC_MUR : dmr::BC_CFB;
+      N.crow = P.crow; N.frow = P.frow;
+      restr_bounds(&N.jlo, &N.jhi, &N.ilo, &N.ihi);
+      N.rinv = (T)(1.0 / (double)cfg.r);
+      for (int k = 1; k <= cfg.r; ++k) N.frac[k] = (T)((double)k / (double)cfg.r);
+      cudaLaunchConfig_t lc = {};
+      multi_config(&lc, la, kNearBlocks, P.nwarps, P.nsmem, kNearBlocks, pdl && !both);
+      if (both) lc.stream = st_near;
+      if (int s = ck(cudaLaunchKernelEx(&lc, near_kernels()[P.nk].f, A, N), "near-region launch")) return s;
+      counted(1);
+    }
+    if (P.tk >= 0) {
+      cudaLaunchConfig_t lc = {};
+      multi_config(&lc, la, P.tiles, P.twarps, P.tsmem, 0, pdl && !both);
+      if (int s = ck(cudaLaunchKernelEx(&lc, tile_kernels()[P.tk].f, A), "tile launch")) return s;
+      counted(1);
+    }
+    if (both) {
+      if (int s = ck(cudaEventRecord(ev_join, st_near), "join")) return s;
+      if (int s = ck(cudaStreamWaitEvent(st, ev_join, 0), "join")) return s;
+    }
+    last_em = !both;   // a launch that follows a join is an ordinary one
+    return DMR_OK;
+  }
+
+  // Coarse steps of the next launch, with `left` steps of the period to go
+  // before the caller's end: equal groups of at most K steps (0: strips).
+  // K without the autotuner: 4 for a uniform mesh (1024^2 per step: 11.3 us at
+  // K = 2, 7.0 at 4, 6.9 at 8, 8.1 at 12, where the halos take over), 8 beside a
+  // near region (512^2: 5.3 us per step at K = 4, 4.4 at 8, 4.4 at 12).
+  int multi_steps(int64_t left) {
+    if (!multi_allowed() || left < 2) return 0;
+    int K = multi_k;
+    if (K == 0) {
+      const MultiPlan& W = multi_get(2);
+      if (!W.ok) return 0;
+      K = W.tk < 0 ? cfg.steps_per_period / 2 : (W.nk < 0 ? 4 : 8);
+      if (K < 2) K = 2;
+    }
+    int64_t g = (left + K - 1) / K;
+    // an even number of launches in a whole period: a captured period then
+    // ends in the buffer parity it starts with
+    if (left == cfg.steps_per_period && (g & 1) && cfg.steps_per_period % 2 == 0) ++g;
+    const int k = (int)((left + g - 1) / g);
+    return multi_get(k).ok ? k : 0;
+  }
+
+  // the coarse steps from level mlev on, `left` of them at most to the next
+  // stop; *done: steps launched
+  int launch_steps(int64_t mlev, int64_t left, int* done) {
+    const int k = multi_steps(left);
+    if (k == 0) {
+      *done = 1;
+      return launch_coarse_step(mlev);
+    }
+    const int fd = fpar ^ (int)(((int64_t)k * cfg.r) & 1);
+    if (int s = go_multi(multi_get(k), mlev, cpar, fpar, fd, pdl_next())) return s;
+    flip_coarse();
+    if (has_fine) {
+      if (fd != fpar) flip_fine();
+      rvalid = true;
+    }
+    *done = k;
+    return launched("multi-step EM");
+  }
+
   // continuity step, totals and flags at the end of a period (coarse level
   // mlev): three launches over the coarse mesh's and the fine rectangle's
   // node tiles (rates, new density, commit with flags and FP64 totals)
@@ -1126,6 +1396,9 @@ struct Engine final : Base {
   dmr::Ctl* hctl = nullptr;
   ~Engine() override {
     if (hctl) cudaFreeHost(hctl);
+    if (st_near) cudaStreamDestroy(st_near);
+    if (ev_fork) cudaEventDestroy(ev_fork);
+    if (ev_join) cudaEventDestroy(ev_join);
   }
   int period_end_host(bool graph_ran = false) {
     if (!hctl)
@@ -1262,8 +1535,8 @@ struct Engine final : Base {
         launches += graph_nodes;
         m += NT;
         n -= NT;
-        if (NT & 1) flip_coarse();
-        if (has_fine && (((int64_t)cfg.r * NT) & 1)) flip_fine();
+        if (g_cend != cpar) flip_coarse();
+        if (has_fine && g_fend != fpar) flip_fine();
         if (has_fine) rvalid = true;
         if (int s = period_end_host(true)) return s;
         continue;
@@ -1281,9 +1554,10 @@ struct Engine final : Base {
         if (int s = period_end_host()) return s;
         continue;
       }
-      if (int s = launch_coarse_step(m)) return s;
-      ++m;
-      --n;
+      int done = 0;
+      if (int s = launch_steps(m, std::min<int64_t>(n, NT - m % NT), &done)) return s;
+      m += done;
+      n -= done;
       if (m % NT == 0) {
         if (int s = launch_period_end(m)) return s;
         if (int s = period_end_host()) return s;
@@ -1314,10 +1588,12 @@ struct Engine final : Base {
       s = go_period();
       if (!s) after_period();
     } else {
-      for (int q = 0; q < NT && !s; ++q) s = launch_coarse_step(m + q);
+      for (int q = 0, done = 0; q < NT && !s; q += done) s = launch_steps(m + q, NT - q, &done);
     }
     if (!s) s = launch_period_end(m + NT);
     capturing = false;
+    g_cend = cpar;
+    g_fend = fpar;
     if (cpar != c0) flip_coarse();
     if (has_fine && fpar != f0) flip_fine();
     rvalid = rv0;
@@ -2140,10 +2416,12 @@ struct Engine final : Base {
   void set_shape(int wps) override {
     warps_per_sm = wps;
     warps_per_sm_fine = wps;
+    strips = true;
     drop_graph();
   }
   void set_cols(int cols) override {
     lanecols = cols;
+    strips = true;
     drop_graph();
   }
   void get_shape(int32_t* out) const override {
@@ -2180,6 +2458,7 @@ struct Engine final : Base {
       if (ms < best) { best = ms; best_w = cand[c]; }
     }
     warps_per_sm = best_w;
+    double strip_ms = best;       // per coarse step
     if (has_fine && cfg.r >= 2) {
       // The coarse step's launches as they run: the merged launch, then fine
       // sub-steps 2..r (each reading the present fine state, writing
@@ -2230,12 +2509,52 @@ struct Engine final : Base {
       warps_per_sm_fine = bf;
       lanecols = blc;
       best_w = bc;
+      strip_ms = best_p / (kTrialLaunches / 2);
       if (int s_ = ck(cudaMemcpyAsync(fS2[cur], fS2[cur ^ 1], s2b, cudaMemcpyDeviceToDevice, st),
                       "autotune: restore S2")) return s_;
     }
+    if (int s_ = autotune_multi(strip_ms)) return s_;
     drop_graph();
     if (wps_out) *wps_out = best_w;
     return launched("autotune");
+  }
+
+  // Coarse steps per launch: K = 4 and 8 (groups of launches as they run, from
+  // the present state into the other buffers; the E^2 sums are kept
+  // aside) against strip_ms per coarse step of the tuned strips.  Strips stay
+  // unless a K is more than 1 % faster.
+  int autotune_multi(double strip_ms) {
+    multi_k = 0;
+    if (!multi_allowed() || multi_steps(cfg.steps_per_period) == 0 || multi_get(2).tk < 0) return DMR_OK;
+    const size_t cs2 = L.cplane * sizeof(double);
+    const size_t fs2 = has_fine ? (size_t)(F[cur].ny + 1) * (size_t)F[cur].p * sizeof(double) : 0;
+    if (int s_ = ck(cudaMemcpyAsync(view, C.S2, cs2, cudaMemcpyDeviceToDevice, st), "keep S2")) return s_;
+    if (has_fine)
+      if (int s_ = ck(cudaMemcpyAsync(fS2[cur ^ 1], fS2[cur], fs2, cudaMemcpyDeviceToDevice, st), "keep S2")) return s_;
+    double best = strip_ms * 0.99;
+    int best_k = 1;
+    for (int K : {4, 8}) {
+      if (K > cfg.steps_per_period || !multi_get(K).ok) continue;
+      int err = DMR_OK;
+      float ms = 0.f;
+      const int reps = 2;
+      auto launch = [&]() {
+        for (int q = 0; q < reps && !err; ++q)
+          err = go_multi(multi_get(K), m, cpar, fpar, fpar ^ 1, q > 0 && pdl_next());
+      };
+      const int64_t l0 = launches;
+      int s_ = ck(graph_time(st, launch, 1, &ms), "autotune trial (several steps)");
+      launches = l0 + 4 * (launches - l0);
+      if (s_ || err) return s_ ? s_ : err;
+      const double per = (double)ms / ((double)reps * K);
+      if (per < best) { best = per; best_k = K; }
+    }
+    multi_k = best_k;
+    last_em = false;
+    if (int s_ = ck(cudaMemcpyAsync(C.S2, view, cs2, cudaMemcpyDeviceToDevice, st), "restore S2")) return s_;
+    if (has_fine)
+      if (int s_ = ck(cudaMemcpyAsync(fS2[cur], fS2[cur ^ 1], fs2, cudaMemcpyDeviceToDevice, st), "restore S2")) return s_;
+    return DMR_OK;
   }
 
   // Measured duration of one EM launch form of the present step, as CUDA-graph
