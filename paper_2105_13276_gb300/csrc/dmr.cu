@@ -9,6 +9,7 @@
 #include <cstdio>
 #include <cstring>
 #include <functional>
+#include <memory>
 #include <new>
 #include <string>
 #include <vector>
@@ -1214,11 +1215,10 @@ struct Engine final : Base {
     lc->numAttrs = (unsigned)n;
   }
 
-  // Launch P.K coarse steps from level mlev: coarse parity cp to cp ^ 1, fine
-  // parity fp to fd.  Tiles on the run's stream, the near region beside them
-  // on a stream of its own that starts and ends with them.
-  int go_multi(const MultiPlan& P, int64_t mlev, int cp, int fp, int fd, bool pdl) {
-    dmr::MultiArgs<T> A{};
+  // Arguments of P.K coarse steps from level mlev: coarse parity cp to cp ^ 1,
+  // fine parity fp to fd.
+  void multi_args(const MultiPlan& P, int64_t mlev, int cp, int fp, int fd, dmr::MultiArgs<T>* A,
+                  dmr::NearArgs<T>* N) const {
     auto mesh = [&](dmr::MultiMesh<T>* M, const dmr::Mesh<T>& m, int rr, int64_t level) {
       M->m = m;
       M->c = make_step(rr, level, true);
@@ -1229,11 +1229,35 @@ struct Engine final : Base {
     };
     dmr::Mesh<T> src = C;
     src.Ex = cE[cp][0]; src.Ey = cE[cp][1]; src.Hz = cE[cp][2]; src.vx = cE[cp][3]; src.vy = cE[cp][4];
-    mesh(&A.C, src, 1, mlev);
-    for (int q = 0; q < 5; ++q) A.C.d[q] = cE[cp ^ 1][q];
-    A.K = P.K;
-    A.hx = P.hx; A.tw = P.tw; A.th = P.th; A.gx = P.gx; A.gy = P.gy;
-    A.z0 = P.zone[0]; A.z1 = P.zone[1]; A.z2 = P.zone[2]; A.z3 = P.zone[3];
+    mesh(&A->C, src, 1, mlev);
+    for (int q = 0; q < 5; ++q) A->C.d[q] = cE[cp ^ 1][q];
+    A->K = P.K;
+    A->hx = P.hx; A->tw = P.tw; A->th = P.th; A->gx = P.gx; A->gy = P.gy;
+    A->z0 = P.zone[0]; A->z1 = P.zone[1]; A->z2 = P.zone[2]; A->z3 = P.zone[3];
+    if (P.nk < 0) return;
+    mesh(&N->F, fine_at(fp), cfg.r, (int64_t)cfg.r * mlev);
+    for (int q = 0; q < 5; ++q) N->F.d[q] = fineE(cur, fd, q);
+    N->r = cfg.r;
+    N->restr = d.coupling == 0;
+    N->I0 = rect[0]; N->J0 = rect[1]; N->I1 = rect[2]; N->J1 = rect[3];
+    N->wi = P.win[0]; N->wj = P.win[1]; N->wnx = P.win[2] - P.win[0]; N->wny = P.win[3] - P.win[1];
+    N->cmode[dmr::SIDE_LEFT] = P.win[0] == 0 ? dmr::BC_MUR : dmr::BC_FROZEN;
+    N->cmode[dmr::SIDE_BOTTOM] = P.win[1] == 0 ? dmr::BC_MUR : dmr::BC_FROZEN;
+    N->cmode[dmr::SIDE_RIGHT] = P.win[2] == cfg.nx ? dmr::BC_MUR : dmr::BC_FROZEN;
+    N->cmode[dmr::SIDE_TOP] = P.win[3] == cfg.ny ? dmr::BC_MUR : dmr::BC_FROZEN;
+    for (int q = 0; q < 4; ++q) N->fmode[q] = side_on_edge(q) ? dmr::BC_MUR : dmr::BC_CFB;
+    N->crow = P.crow; N->frow = P.frow;
+    restr_bounds(&N->jlo, &N->jhi, &N->ilo, &N->ihi);
+    N->rinv = (T)(1.0 / (double)cfg.r);
+    for (int k = 1; k <= cfg.r; ++k) N->frac[k] = (T)((double)k / (double)cfg.r);
+  }
+
+  // Launch P.K coarse steps (multi_args).  Tiles on the run's stream, the near
+  // region beside them on a stream of its own that starts and ends with them.
+  int go_multi(const MultiPlan& P, int64_t mlev, int cp, int fp, int fd, bool pdl) {
+    dmr::MultiArgs<T> A{};
+    dmr::NearArgs<T> N{};
+    multi_args(P, mlev, cp, fp, fd, &A, &N);
     const bool both = P.nk >= 0 && P.tk >= 0;
     if (both) {
       if (!st_near) {
@@ -1248,22 +1272,6 @@ struct Engine final : Base {
     }
     cudaLaunchAttribute la[2];
     if (P.nk >= 0) {
-      dmr::NearArgs<T> N{};
-      mesh(&N.F, fine_at(fp), cfg.r, (int64_t)cfg.r * mlev);
-      for (int q = 0; q < 5; ++q) N.F.d[q] = fineE(cur, fd, q);
-      N.r = cfg.r;
-      N.restr = d.coupling == 0;
-      N.I0 = rect[0]; N.J0 = rect[1]; N.I1 = rect[2]; N.J1 = rect[3];
-      N.wi = P.win[0]; N.wj = P.win[1]; N.wnx = P.win[2] - P.win[0]; N.wny = P.win[3] - P.win[1];
-      N.cmode[dmr::SIDE_LEFT] = P.win[0] == 0 ? dmr::BC_MUR : dmr::BC_FROZEN;
-      N.cmode[dmr::SIDE_BOTTOM] = P.win[1] == 0 ? dmr::BC_MUR : dmr::BC_FROZEN;
-      N.cmode[dmr::SIDE_RIGHT] = P.win[2] == cfg.nx ? dmr::BC_MUR : dmr::BC_FROZEN;
-      N.cmode[dmr::SIDE_TOP] = P.win[3] == cfg.ny ? dmr::BC_MUR : dmr::BC_FROZEN;
-      for (int q = 0; q < 4; ++q) N.fmode[q] = side_on_edge(q) ? dmr::BC_MUR : dmr::BC_CFB;
-      N.crow = P.crow; N.frow = P.frow;
-      restr_bounds(&N.jlo, &N.jhi, &N.ilo, &N.ihi);
-      N.rinv = (T)(1.0 / (double)cfg.r);
-      for (int k = 1; k <= cfg.r; ++k) N.frac[k] = (T)((double)k / (double)cfg.r);
       cudaLaunchConfig_t lc = {};
       multi_config(&lc, la, kNearBlocks, P.nwarps, P.nsmem, kNearBlocks, pdl && !both);
       if (both) lc.stream = st_near;
@@ -2877,6 +2885,126 @@ struct Batch final : BatchBase {
     return 1;
   }
 
+  // ---- several coarse steps per launch (dmr_multi.cuh): the whole periods of
+  // FP32 runs that all have a near region.  One launch of tiles and one of
+  // near regions (a cluster per run) per K steps and kMultiRuns runs, side by
+  // side on two streams.  k_em_batch holds 94 registers (its arguments come
+  // from shared memory) and streams each step's state: 16 runs of 128^2 to
+  // 1024^2, 7.6 M nodes, took 142 us per coarse step, 79 us here.
+  struct MultiBatchPlan {
+    bool ok = false;
+    int K = 0, twarps = 0, nk = 0, nwarps = 0;
+    size_t tsmem = 0, nsmem = 0;
+    std::vector<typename Engine<T>::MultiPlan> run;
+  };
+  MultiBatchPlan multi_plan() {
+    MultiBatchPlan P;
+    if constexpr (sizeof(T) == 4) {
+      double nodes = 0.0;
+      int rows = 1 << 30;
+      for (auto* e : runs) {
+        if (!e->has_fine || e->strips || e->timing || e->cfg.nx + 1 < 32 * Engine<T>::kMC) return P;
+        nodes += (double)(e->cfg.nx + 1) * (e->cfg.ny + 1);
+        rows = std::min(rows, e->cfg.ny + 1);
+      }
+      // long halos where launches count, short ones where the nodes do
+      P.K = std::min(NT / 2, nodes > 1e6 ? 4 : 8);
+      if (P.K < 2) return P;
+      for (auto* e : runs) {
+        P.run.push_back(e->multi_plan(P.K));
+        if (!P.run.back().ok || P.run.back().nk < 0) return P;
+        P.nk = std::max(P.nk, P.run.back().nk);
+        P.nsmem = std::max(P.nsmem, P.run.back().nsmem);
+      }
+      const int R = Engine<T>::tile_kernels()[0].R, NR = Engine<T>::near_kernels()[P.nk].R;
+      for (size_t q = 0; q < runs.size(); ++q) {
+        auto& p = P.run[q];
+        const auto* e = runs[q];
+        const int fcols = e->cfg.r * (e->rect[2] - e->rect[0]) + 1, ccols = p.win[2] - p.win[0] + 1;
+        P.nwarps = std::max(P.nwarps, dmr::near_units(fcols, p.frow + 1, NR) + dmr::near_units(ccols, p.crow + 1, NR));
+      }
+      // rows per tile: the fewest rows that the busiest SM has to step
+      double best = 1e300;
+      for (int w = 8; w <= 32; ++w) {
+        const int H = w * R, th = H - 2 * P.K;
+        if (th < 1 || H > rows) continue;
+        long long tiles = 0;
+        for (size_t q = 0; q < runs.size(); ++q)
+          if (P.run[q].tk >= 0) tiles += (long long)P.run[q].gx * ((runs[q]->cfg.ny + 1 + th - 1) / th);
+        const double per_sm = w > 16 ? 1.0 : 2.0;
+        const double cost = std::ceil(tiles / (per_sm * runs[0]->num_sms)) * per_sm * H;
+        if (cost < best) { best = cost; P.twarps = w; }
+      }
+      if (P.twarps == 0) return P;
+      P.tsmem = dmr::tile_smem<T, Engine<T>::kMC>(P.twarps, P.K);
+      for (size_t q = 0; q < runs.size(); ++q) {
+        auto& p = P.run[q];
+        if (p.tk < 0) { p.tiles = 0; continue; }
+        p.th = P.twarps * R - 2 * P.K;
+        p.gy = (runs[q]->cfg.ny + 1 + p.th - 1) / p.th;
+        p.tiles = p.gx * p.gy;
+      }
+      auto kt = dmr::k_multi_batch<T, Engine<T>::kMC, 2, 1024>;
+      auto kn = P.nk == 0 ? dmr::k_near_batch<T, 1, 1024> : dmr::k_near_batch<T, 2, 1024>;
+      cudaFuncSetAttribute(kt, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)Engine<T>::kMaxSmem);
+      cudaFuncSetAttribute(kn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)Engine<T>::kMaxSmem);
+      cudaFuncSetAttribute(kn, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+      cudaLaunchConfig_t lc = {};
+      cudaLaunchAttribute la[2];
+      runs[0]->multi_config(&lc, la, Engine<T>::kNearBlocks, P.nwarps, P.nsmem, Engine<T>::kNearBlocks, false);
+      int n = 0;
+      P.ok = P.nsmem + 2048 <= Engine<T>::kMaxSmem &&
+             cudaOccupancyMaxActiveClusters(&n, kn, &lc) == cudaSuccess && n > 0;
+      if (!P.ok) cudaGetLastError();
+    }
+    return P;
+  }
+
+  // a whole period's coarse steps from level m0, host parities cp; launches counted in *nl
+  int launch_multi(const MultiBatchPlan& P, int64_t m0, int64_t* nl) {
+    if constexpr (sizeof(T) == 4) {
+      if (side.empty()) return fail(DMR_ESTATE, "no side stream");
+      auto kt = dmr::k_multi_batch<T, Engine<T>::kMC, 2, 1024>;
+      auto kn = P.nk == 0 ? dmr::k_near_batch<T, 1, 1024> : dmr::k_near_batch<T, 2, 1024>;
+      int groups = (NT + P.K - 1) / P.K;
+      groups += groups & 1;              // an even number: the buffer parity comes back
+      auto B = std::make_unique<dmr::MultiBatch<T>>();
+      int done = 0;
+      for (int g = 0; g < groups; ++g) {
+        const int k = (NT - done + groups - g - 1) / (groups - g);
+        cudaEventRecord(fork, st);
+        cudaStreamWaitEvent(side[0], fork, 0);
+        for (size_t q0 = 0; q0 < runs.size(); q0 += dmr::kMultiRuns) {
+          const int n = (int)std::min<size_t>(dmr::kMultiRuns, runs.size() - q0);
+          B->nruns = n;
+          B->off[0] = 0;
+          for (int q = 0; q < n; ++q) {
+            auto p = P.run[q0 + q];
+            p.K = k;
+            runs[q0 + q]->multi_args(p, m0 + done, g & 1, 0, 0, &B->a[q], &B->n[q]);
+            B->off[q + 1] = B->off[q] + p.tiles;
+          }
+          cudaLaunchConfig_t lc = {};
+          cudaLaunchAttribute la[2];
+          runs[0]->multi_config(&lc, la, n * Engine<T>::kNearBlocks, P.nwarps, P.nsmem, Engine<T>::kNearBlocks, false);
+          lc.stream = side[0];
+          if (int s = ck(cudaLaunchKernelEx(&lc, kn, *B), "near-region launch")) return s;
+          ++*nl;
+          if (B->off[n] == 0) continue;
+          cudaLaunchConfig_t lt = {};
+          runs[0]->multi_config(&lt, la, B->off[n], P.twarps, P.tsmem, 0, false);
+          lt.stream = st;
+          if (int s = ck(cudaLaunchKernelEx(&lt, kt, *B), "tile launch")) return s;
+          ++*nl;
+        }
+        cudaEventRecord(join[0], side[0]);
+        cudaStreamWaitEvent(st, join[0], 0);
+        done += k;
+      }
+    }
+    return DMR_OK;
+  }
+
   // EM launches of coarse step q of the period starting at level m0
   int launch_step(int64_t m0, int q, bool first) {
     const int cp = (int)((m0 + q) & 1);
@@ -2940,7 +3068,10 @@ struct Batch final : BatchBase {
     if (int s = ck(cudaStreamBeginCapture(st, cudaStreamCaptureModeThreadLocal), "begin capture")) return s;
     int s = DMR_OK;
     graph_nodes = 0;
-    for (int q = 0; q < NT; ++q) graph_nodes += launch_step(m, q, q == 0 && first_pending);
+    const MultiBatchPlan P = multi_plan();
+    if (P.ok) s = launch_multi(P, m, &graph_nodes);
+    else
+      for (int q = 0; q < NT; ++q) graph_nodes += launch_step(m, q, q == 0 && first_pending);
     // period ends: one parallel branch per run
     cudaEventRecord(fork, st);
     std::vector<bool> rv(runs.size());

@@ -873,4 +873,44 @@ __global__ void __launch_bounds__(TH) k_near(MultiArgs<T> A, NearArgs<T> N) {
   multi_near<T, R>(A, N, multi_smem);
 }
 
+// The same for the runs of a batch: their arguments in the launch's parameters
+// (a block copies its run's into shared memory), tiles of run q from block
+// off[q] on, one cluster per run.
+constexpr int kMultiRuns = 40;
+template <class T>
+struct MultiBatch {
+  int nruns, off[kMultiRuns + 1];
+  MultiArgs<T> a[kMultiRuns];
+  NearArgs<T> n[kMultiRuns];
+};
+static_assert(sizeof(MultiBatch<float>) <= 32764, "kernel parameters");
+
+template <class A>
+__device__ __forceinline__ void multi_stage(A* dst, const A& src) {
+  static_assert(sizeof(A) % 4 == 0, "words");
+  const int* s = reinterpret_cast<const int*>(&src);
+  for (int q = threadIdx.x; q < (int)(sizeof(A) / 4); q += blockDim.x) reinterpret_cast<int*>(dst)[q] = s[q];
+}
+
+template <class T, int C, int R, int TH>
+__global__ void __launch_bounds__(TH) k_multi_batch(const __grid_constant__ MultiBatch<T> B) {
+  __shared__ MultiArgs<T> A;
+  int q = 0;
+  while (q + 1 < B.nruns && (int)blockIdx.x >= B.off[q + 1]) ++q;
+  multi_stage(&A, B.a[q]);
+  __syncthreads();
+  multi_tiles<T, C, R>(A, (int)blockIdx.x - B.off[q], reinterpret_cast<T*>(multi_smem));
+}
+
+template <class T, int R, int TH>
+__global__ void __launch_bounds__(TH) k_near_batch(const __grid_constant__ MultiBatch<T> B) {
+  __shared__ MultiArgs<T> A;
+  __shared__ NearArgs<T> N;
+  const int q = (int)blockIdx.x / cluster_size();
+  multi_stage(&A, B.a[q]);
+  multi_stage(&N, B.n[q]);
+  __syncthreads();
+  multi_near<T, R>(A, N, multi_smem);
+}
+
 }  // namespace dmr

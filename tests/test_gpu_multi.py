@@ -114,3 +114,31 @@ def test_growth_in_free_running_mode():
             for f in FIELDS:
                 assert np.array_equal(runs[0].read(f, level), runs[1].read(f, level)), (f, level)
     assert len(grown) > 1
+
+
+def test_batch_of_more_runs_than_one_launch_takes():
+    """43 runs of uneven sizes (40 per launch): each has the bits of its own run
+    with one launch per step; whole periods in groups, the rest step by step."""
+    rng = np.random.default_rng(5)
+    sizes = [(int(rng.integers(63, 170)), int(rng.integers(60, 150))) for _ in range(43)]
+    cfgs, rects = [], []
+    for nx, ny in sizes:
+        cfgs.append(W.base_cfg(nx=nx, ny=ny, r=2, n_lambda=16, steps_per_period=32, precision=1, growth=0,
+                               E0=float(rng.uniform(3e6, 6e6)), coupling=int(rng.integers(0, 2))))
+        i0, j0 = int(rng.integers(0, nx - 12)), int(rng.integers(0, ny - 9))
+        rects.append((i0, j0, i0 + 12, j0 + 9))
+    batch = D.Batch(cfgs)
+    for run, rect in zip(batch.runs, rects):
+        run.set_patch(rect)
+        run.seed_gaussian(3e17, rect[0] * run.dxc, rect[1] * run.dxc, 0.1 * run.lam, 0.1 * run.lam)
+    batch.advance(64)
+    batch.advance(5)
+    for q in (0, 17, 39, 40, 42):
+        one = D.Run(cfgs[q])
+        one.set_launch_shape(48)
+        one.set_patch(rects[q])
+        one.seed_gaussian(3e17, rects[q][0] * one.dxc, rects[q][1] * one.dxc, 0.1 * one.lam, 0.1 * one.lam)
+        one.advance(69)
+        for level in (0, 1):
+            for f in FIELDS:
+                assert np.array_equal(batch.runs[q].read(f, level), one.read(f, level)), (q, f, level)
