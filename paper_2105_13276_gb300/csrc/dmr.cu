@@ -1661,6 +1661,28 @@ struct Engine final : Base {
     }
   }
 
+  // Rows of cols elements from src (pitch sp elements) to dst (pitch dp) on the
+  // run's stream.  user: the caller's device buffer; one that is this device's
+  // memory and aligned to its elements is copied by a kernel, anything else by
+  // the runtime (which also refuses what is not a device pointer).
+  int copy2d(void* dst, int dp, const void* src, int sp, int cols, int rows, int es, const void* user,
+             cudaMemcpyKind kind, const char* what) {
+    cudaPointerAttributes at{};
+    int dev = -1;
+    if (user && (es == 4 || es == 8) && (uintptr_t)user % es == 0 && cudaGetDevice(&dev) == cudaSuccess &&
+        cudaPointerGetAttributes(&at, user) == cudaSuccess && at.type == cudaMemoryTypeDevice && at.device == dev) {
+      const dim3 g((cols + dmr::kCopyX * dmr::kCopyU - 1) / (dmr::kCopyX * dmr::kCopyU),
+                   (rows + dmr::kCopyY - 1) / dmr::kCopyY);
+      const dim3 b(dmr::kCopyX, dmr::kCopyY);
+      if (es == 4) dmr::k_copy2d<float><<<g, b, 0, st>>>((float*)dst, dp, (const float*)src, sp, cols, rows);
+      else dmr::k_copy2d<double><<<g, b, 0, st>>>((double*)dst, dp, (const double*)src, sp, cols, rows);
+      counted(1);
+      return launched("field copy");
+    }
+    cudaGetLastError();
+    return ck(cudaMemcpy2DAsync(dst, (size_t)dp * es, src, (size_t)sp * es, (size_t)cols * es, rows, kind, st), what);
+  }
+
   int read(int field, int level, void* dst, size_t bytes, int dev) override {
     int rows, cols, es;
     if (int s = dims(field, level, &rows, &cols, &es)) return fail(s, "no such field / level");
@@ -1693,10 +1715,8 @@ struct Engine final : Base {
       if (int e = launched("E_rms view")) return e;
       src = view;
     }
-    const size_t wb = (size_t)cols * es;
-    cudaError_t e = cudaMemcpy2DAsync(dst, wb, src, (size_t)p * es, wb, rows,
-                                      dev ? cudaMemcpyDeviceToDevice : cudaMemcpyDeviceToHost, st);
-    if (int s = ck(e, "cudaMemcpy2DAsync(read)")) return s;
+    if (int s = copy2d(dst, cols, src, p, cols, rows, es, dev ? dst : nullptr,
+                       dev ? cudaMemcpyDeviceToDevice : cudaMemcpyDeviceToHost, "cudaMemcpy2DAsync(read)")) return s;
     if (!dev) return ck(cudaStreamSynchronize(st), "read sync");
     return DMR_OK;
   }
@@ -1708,10 +1728,8 @@ struct Engine final : Base {
     if (int s = dims(field, level, &rows, &cols, &es)) return fail(s, "no such field / level");
     if (bytes < (size_t)rows * cols * es) return fail(DMR_ECAPACITY, "source too small");
     const int p = level == 0 ? C.p : F[cur].p;
-    const size_t wb = (size_t)cols * es;
-    cudaError_t e = cudaMemcpy2DAsync(field_ptr(field, level), (size_t)p * es, src, wb, wb, rows,
-                                      dev ? cudaMemcpyDeviceToDevice : cudaMemcpyHostToDevice, st);
-    if (int s = ck(e, "cudaMemcpy2DAsync(write)")) return s;
+    if (int s = copy2d(field_ptr(field, level), p, src, cols, cols, rows, es, dev ? src : nullptr,
+                       dev ? cudaMemcpyDeviceToDevice : cudaMemcpyHostToDevice, "cudaMemcpy2DAsync(write)")) return s;
     if (field == DMR_FIELD_NE && level == 1) inject();
     if (!dev) return ck(cudaStreamSynchronize(st), "write sync");
     return launched("write");

@@ -1711,13 +1711,29 @@ __global__ void k_erms_view(Mesh<T> m, Step<T> c, double q, T* out) {
   out[j * m.p + i] = (T)sqrt(s2 / q);
 }
 
-// strided 2-D copy between a dense buffer and a pitched array (device side)
+// Strided 2-D copy between a dense buffer and a pitched array on the device:
+// kCopyX * kCopyU columns of kCopyY rows per block, the loads of a thread's
+// elements all in flight.  A dense buffer's rows start anywhere (an odd number
+// of columns), so the accesses are single elements, 128 bytes per warp.  Six
+// fields of both meshes of a 2048 x 1024 run at r = 4 (252 MB): 129 us, with
+// cudaMemcpy2DAsync 304 us; of a 1024 x 1024 mesh 25 against 50 us; at 512 x 512
+// and below the call costs what it did.
+constexpr int kCopyX = 128, kCopyY = 4, kCopyU = 4;
 template <class E>
-__global__ void k_copy2d(E* dst, int dp, const E* src, int sp, int cols, int rows) {
-  const int i = blockIdx.x * blockDim.x + threadIdx.x;
-  const int j = blockIdx.y * blockDim.y + threadIdx.y;
-  if (i >= cols || j >= rows) return;
-  dst[(size_t)j * dp + i] = src[(size_t)j * sp + i];
+__global__ void __launch_bounds__(kCopyX* kCopyY) k_copy2d(E* __restrict__ dst, int dp, const E* __restrict__ src, int sp,
+                                                            int cols, int rows) {
+  const int i = blockIdx.x * (kCopyX * kCopyU) + threadIdx.x;
+  const int j = blockIdx.y * kCopyY + threadIdx.y;
+  if (j >= rows) return;
+  const E* s = src + (size_t)j * sp;
+  E* d = dst + (size_t)j * dp;
+  E v[kCopyU];
+#pragma unroll
+  for (int u = 0; u < kCopyU; ++u)
+    if (i + u * kCopyX < cols) v[u] = s[i + u * kCopyX];
+#pragma unroll
+  for (int u = 0; u < kCopyU; ++u)
+    if (i + u * kCopyX < cols) d[i + u * kCopyX] = v[u];
 }
 
 }  // namespace dmr
