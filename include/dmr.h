@@ -286,8 +286,9 @@ int dmr_sync(const dmr_ctx* ctx);
  * combination is also timed with two node columns per lane in sub-steps
  * 2..r (dmr_set_strip_columns); two must be more than 1 % faster to be
  * chosen.  Last, FP32 runs with Mur sides time groups of launches that advance
- * 4 and 8 coarse steps each, and take them where they are more than 1 % faster
- * per coarse step.  *warps_per_sm returns the merged launch's choice
+ * 4 and 8 coarse steps each, and runs without them the coarse step's launch
+ * with one launch of all r fine sub-steps; each is taken where it is more than
+ * 1 % faster per coarse step.  *warps_per_sm returns the merged launch's choice
  * (dmr_get_launch_shape gives the whole shape). */
 int dmr_autotune(dmr_ctx* ctx, int32_t* warps_per_sm, double trial_ms[5]);
 

@@ -1034,6 +1034,16 @@ struct Engine final : Base {
       return launched("coarse EM");
     }
     const int cp0 = cpar;
+    if (fine_allowed() && fine_plan().ok) {
+      go_em(Ac.nblk + Ac.ncfb, Ac, pdl_next());
+      last_em = true;
+      flip_coarse();
+      if (int s = go_fine(fine_plan(), mlev, cp0, fpar, pdl_next())) return s;
+      counted(2);
+      flip_fine();
+      rvalid = true;
+      return launched("EM step");
+    }
     const double fn = (double)(F[cur].nx + 1) * (F[cur].ny + 1);
     for (int k = 1; k <= r; ++k) {
       const int64_t mf = (int64_t)r * mlev + (k - 1);
@@ -1075,6 +1085,23 @@ struct Engine final : Base {
   static std::vector<NearKernel> near_kernels() {
     if constexpr (sizeof(T) == 4) return {{1, 1024, dmr::k_near<T, 1, 1024>}, {2, 1024, dmr::k_near<T, 2, 1024>}};
     else return {};
+  }
+  // What a launch of `tiles` tiles of H rows costs, w warps each on sms SMs: the
+  // rows that the busiest SM steps, times what a row costs where n blocks
+  // share it (one's loads and stores overlap another's steps; 1024^2 at K = 4,
+  // relative: 2.9 for one block per SM, 2.4, 2.0 and 1.8 for two, three, four).
+  double tile_cost(int q, int w, size_t smem, long long tiles, int H, int sms) const {
+    int per_sm = 0;
+    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, tile_kernels()[q].f, 32 * w, smem) != cudaSuccess ||
+        per_sm < 1) {
+      cudaGetLastError();
+      return 1e300;
+    }
+    per_sm = std::min(per_sm, 4);
+    const double f[5] = {0.0, 2.9, 2.4, 2.0, 1.8};
+    const int n = (int)std::min<long long>(per_sm, (tiles + sms - 1) / sms);
+    const long long rounds = (tiles + (long long)sms * n - 1) / ((long long)sms * n);
+    return (double)rounds * n * H * f[std::max(n, 1)];
   }
   struct MultiPlan {
     int K = 0;             // coarse steps per launch
@@ -1154,7 +1181,7 @@ struct Engine final : Base {
     P.tw = W - 2 * P.hx;
     if (P.tw < 8 || nx + 1 < W) return P;
     P.gx = (nx + 1 + P.tw - 1) / P.tw;
-    // the kernel and the rows per tile: the fewest rows that the busiest SM has to step
+    // the kernel and the rows per tile (tile_cost)
     const int sms = std::max(1, num_sms - (has_fine ? kNearBlocks : 0));
     double best = 1e300;
     const auto kt = tile_kernels();
@@ -1163,7 +1190,7 @@ struct Engine final : Base {
         const int H = w * kt[q].R, th = H - 2 * K;
         if (th < 1 || H > ny + 1) continue;
         const int tiles = P.gx * ((ny + 1 + th - 1) / th);
-        const double cost = (double)((tiles + sms - 1) / sms) * H;
+        const double cost = tile_cost((int)q, w, dmr::tile_smem<T, kMC>(w, K), tiles, H, sms);
         if (cost >= best) continue;
         best = cost;
         P.tk = (int)q;
@@ -1290,6 +1317,93 @@ struct Engine final : Base {
     }
     last_em = !both;   // a launch that follows a join is an ordinary one
     return DMR_OK;
+  }
+
+  // ---- the fine sub-steps of a coarse step in one launch (k_fine) ----------
+  struct FinePlan {
+    bool ok = false;
+    int rect[4] = {-1, -1, -1, -1};
+    int tk = 0, warps = 0, tiles = 0, tw = 0, th = 0, gx = 0, gy = 0, hx = 0;
+    size_t smem = 0;
+  } fplan;
+  int fine_tiles = 0;      // 0: by rule (r >= 3), 1: no, 2: yes (the autotuner's choice)
+  using FineKernel = void (*)(dmr::MultiArgs<T>, dmr::FineArgs<T>);
+  static FineKernel fine_kernel(int tk) {
+    if constexpr (sizeof(T) == 4) return tk == 0 ? dmr::k_fine<T, kMC, 2, 1024> : dmr::k_fine<T, kMC, 4, 512>;
+    else return nullptr;
+  }
+  // All r sub-steps in one launch of tiles, after the coarse step's: FP32, a
+  // fine mesh of a tile at least.
+  const FinePlan& fine_plan() {
+    bool same = true;
+    for (int q = 0; q < 4; ++q) same = same && fplan.rect[q] == rect[q];
+    if (same) return fplan;
+    FinePlan P;
+    for (int q = 0; q < 4; ++q) P.rect[q] = rect[q];
+    const int r = cfg.r, nx = F[cur].nx, ny = F[cur].ny;
+    constexpr int W = 32 * kMC;
+    P.hx = (r + kMC - 1) / kMC * kMC;
+    const int g = r % kMC ? r * kMC : r;             // owned columns: whole coarse cells and lanes
+    P.tw = (W - 2 * P.hx) / g * g;
+    if (P.tw > 0 && nx + 1 >= W) {
+      P.gx = (nx + 1 + P.tw - 1) / P.tw;
+      for (const auto& k : tile_kernels())
+        cudaFuncSetAttribute(k.f, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kMaxSmem);
+      double best = 1e300;
+      const auto kt = tile_kernels();
+      for (size_t q = 0; q < kt.size(); ++q)
+        for (int w = 4; w <= kt[q].TH / 32; ++w) {
+          const int H = w * kt[q].R, th = (H - 2 * r) / r * r;
+          if (th < 1 || H > ny + 1) continue;
+          const int tiles = P.gx * ((ny + 1 + th - 1) / th);
+          const size_t sm = dmr::fine_smem<T, kMC>(w, kt[q].R, r);
+          const double cost = tile_cost((int)q, w, sm, tiles, H, num_sms);
+          if (cost >= best) continue;
+          best = cost;
+          P.tk = (int)q; P.warps = w; P.th = th; P.tiles = tiles; P.gy = tiles / P.gx;
+          P.smem = dmr::fine_smem<T, kMC>(w, kt[q].R, r);
+        }
+      P.ok = P.warps > 0;
+      for (int q = 0; q < 2 && P.ok; ++q)
+        cudaFuncSetAttribute(fine_kernel(q), cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kMaxSmem);
+    }
+    fplan = P;
+    return fplan;
+  }
+  bool fine_allowed() const {
+    return sizeof(T) == 4 && has_fine && !strips && !timing && !in_batch && !persist_on() && fine_tiles != 1 &&
+           (fine_tiles == 2 || cfg.r >= 3);
+  }
+  // sub-steps 1 .. r of coarse step mlev: fine parity fp to fp ^ 1, coarse
+  // levels n, n + 1 in parities cp, cp ^ 1
+  int go_fine(const FinePlan& P, int64_t mlev, int cp, int fp, bool pdl) {
+    dmr::EmArgs<T> Af;
+    em_args_for(cfg.r, mlev, cp, fp, true, nullptr, &Af);   // sides, lines, means
+    dmr::MultiArgs<T> A{};
+    const int64_t mf = (int64_t)cfg.r * mlev;
+    A.C.m = fine_at(fp);
+    for (int q = 0; q < 5; ++q) A.C.d[q] = fineE(cur, fp ^ 1, q);
+    A.C.c = make_step(cfg.r, mf, true);
+    A.C.ps = ph[2]; A.C.pc = ph[3];
+    A.C.N = cfg.r * cfg.steps_per_period;
+    A.C.q0 = (int)(mf % A.C.N);
+    A.K = cfg.r;
+    A.hx = P.hx; A.tw = P.tw; A.th = P.th; A.gx = P.gx; A.gy = P.gy;
+    A.z0 = A.z1 = 1;
+    A.z2 = A.z3 = 0;
+    dmr::FineArgs<T> G{};
+    for (int q = 0; q < 4; ++q) {
+      G.mode[q] = Af.b.mode[q];
+      G.old_line[q] = Af.b.old_line[q]; G.new_line[q] = Af.b.new_line[q];
+      G.stride[q] = Af.b.stride[q]; G.len[q] = Af.b.len[q]; G.start[q] = Af.b.start[q];
+    }
+    G.r = cfg.r;
+    for (int k = 1; k <= cfg.r; ++k) G.frac[k] = (T)((double)k / (double)cfg.r);
+    G.W = Af.W;
+    cudaLaunchConfig_t lc = {};
+    cudaLaunchAttribute la[2];
+    multi_config(&lc, la, P.tiles, P.warps, P.smem, 0, pdl);
+    return ck(cudaLaunchKernelEx(&lc, fine_kernel(P.tk), A, G), "fine tile launch");
   }
 
   // Coarse steps of the next launch, with `left` steps of the period to go
@@ -2539,6 +2653,32 @@ struct Engine final : Base {
       if (int s_ = ck(cudaMemcpyAsync(fS2[cur], fS2[cur ^ 1], s2b, cudaMemcpyDeviceToDevice, st),
                       "autotune: restore S2")) return s_;
     }
+    fine_tiles = 0;
+    if (sizeof(T) == 4 && has_fine && cfg.r >= 2 && !strips && !timing && !in_batch && !persist_on() && fine_plan().ok) {
+      // the coarse step's launch and one of fine tiles, as above (the tiles'
+      // E^2 samples kept aside in the same way)
+      const size_t s2b = (size_t)(F[cur].ny + 1) * (size_t)F[cur].p * sizeof(double);
+      if (int s_ = ck(cudaMemcpyAsync(fS2[cur ^ 1], fS2[cur], s2b, cudaMemcpyDeviceToDevice, st), "autotune: keep S2"))
+        return s_;
+      dmr::EmArgs<T> Ac;
+      em_args_for(1, m, cpar, fpar, true, &Ac, nullptr);
+      int err = DMR_OK;
+      auto launch = [&]() {
+        for (int q = 0; q < kTrialLaunches / 2 && !err; ++q) {
+          go_em(Ac.nblk + Ac.ncfb, Ac, q > 0);
+          err = go_fine(fine_plan(), m, cpar, fpar, true);
+        }
+      };
+      float ms = 0.f;
+      int s_ = ck(graph_time(st, launch, 1, &ms), "autotune trial (fine tiles)");
+      launches += 4 * (int64_t)kTrialLaunches;
+      if (s_ || err) return s_ ? s_ : err;
+      if (int e_ = ck(cudaMemcpyAsync(fS2[cur], fS2[cur ^ 1], s2b, cudaMemcpyDeviceToDevice, st), "autotune: restore S2"))
+        return e_;
+      const double per = (double)ms / (kTrialLaunches / 2);
+      fine_tiles = per < 0.99 * strip_ms ? 2 : 1;
+      strip_ms = std::min(strip_ms, per);
+    }
     if (int s_ = autotune_multi(strip_ms)) return s_;
     drop_graph();
     if (wps_out) *wps_out = best_w;
@@ -2941,7 +3081,7 @@ struct Batch final : BatchBase {
         const int fcols = e->cfg.r * (e->rect[2] - e->rect[0]) + 1, ccols = p.win[2] - p.win[0] + 1;
         P.nwarps = std::max(P.nwarps, dmr::near_units(fcols, p.frow + 1, NR) + dmr::near_units(ccols, p.crow + 1, NR));
       }
-      // rows per tile: the fewest rows that the busiest SM has to step
+      // rows per tile (tile_cost)
       double best = 1e300;
       for (int w = 8; w <= 32; ++w) {
         const int H = w * R, th = H - 2 * P.K;
@@ -2949,8 +3089,7 @@ struct Batch final : BatchBase {
         long long tiles = 0;
         for (size_t q = 0; q < runs.size(); ++q)
           if (P.run[q].tk >= 0) tiles += (long long)P.run[q].gx * ((runs[q]->cfg.ny + 1 + th - 1) / th);
-        const double per_sm = w > 16 ? 1.0 : 2.0;
-        const double cost = std::ceil(tiles / (per_sm * runs[0]->num_sms)) * per_sm * H;
+        const double cost = runs[0]->tile_cost(0, w, dmr::tile_smem<T, Engine<T>::kMC>(w, P.K), tiles, H, runs[0]->num_sms);
         if (cost < best) { best = cost; P.twarps = w; }
       }
       if (P.twarps == 0) return P;

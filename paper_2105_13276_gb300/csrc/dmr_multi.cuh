@@ -13,9 +13,15 @@
 //    the rows next to another warp's through shared memory, one block barrier
 //    per step.  Bound by instruction issue and, for the FP64 E^2 sums, by the
 //    FP64 pipe (16 cycles per warp and SM for an add; a conversion would take as
-//    many, see to_f64).  1024^2: 11.4 us per step with one launch each, 7.0 us
-//    with K = 4 (9.1 us with the conversion instruction); 512^2: 1.8 us of tiles
-//    per step at K = 8.
+//    many, see to_f64).  1024^2: 11.4 us per step with one launch each, 6.1 us
+//    with K = 4 (with one block per SM 7.0 us, and 9.1 us with the conversion
+//    instruction); 512^2: 1.8 us of tiles per step at K = 8.
+//
+//  * Fine tiles (k_fine).  The r sub-steps of a larger fine mesh in one launch of
+//    such tiles after the coarse step's launch; the coarse-fine sides blend the
+//    coarse lines of both levels, the last sub-step writes the fine->coarse
+//    means.  2048 x 1024, a quarter of it refined: 392 us per coarse step at
+//    r = 4 with one launch per sub-step, 211 us here; r = 2: 78 to 62 us.
 //
 //  * The near region (k_near).  The fine rectangle with its r sub-steps per
 //    coarse step and the coarse nodes up to 2K + 1 around it live in one
@@ -89,6 +95,18 @@ struct MultiArgs {
   int z0, z1, z2, z3;  // nodes (i0, j0, i1, j1) the near region stores; z0 > z2: none
 };
 
+// The fine mesh's r sub-steps of one coarse step in tiles (k_fine): its sides,
+// the coarse lines around it (levels n and n + 1) and the fine->coarse means.
+template <class T>
+struct FineArgs {
+  int mode[4];                 // BC_MUR or BC_CFB
+  const T *old_line[4], *new_line[4];
+  int stride[4], len[4], start[4];
+  int r;
+  T frac[17];                  // k / r
+  RestrW<T> W;
+};
+
 // The near region (see above).  Its coarse window is a mesh of its own: nodes
 // [wi, wi + wnx] x [wj, wj + wny], sides Mur where they are the domain's,
 // frozen elsewhere.
@@ -131,12 +149,23 @@ __host__ __device__ constexpr size_t tile_smem(int warps, int K) {
   return ((size_t)2 * 3 * warps + K) * 32 * C * sizeof(T);
 }
 
+template <class T, int C>
+__host__ __device__ constexpr size_t fine_smem(int warps, int R, int K) {
+  const size_t step = tile_smem<T, C>(warps, K) + (size_t)4 * (32 * C + R * warps) * sizeof(T);
+  const size_t means = (size_t)2 * 32 * C * R * warps * sizeof(T);
+  return step > means ? step : means;
+}
+
 // One tile: lane l holds columns ox + C l .., warp w rows oy + R w ... .
 // EDGE: the tile touches a side of the mesh; its origin is then moved inside
 // so that the mesh's first / last row is the tile's first / last row (rows 0,
-// 1 and ny - 1, ny in one thread each, for the Mur sides).
-template <class T, int C, int R, bool EDGE>
-__device__ __forceinline__ void multi_tile(const MultiArgs<T>& A, int bx, int by, int ox, int oy, T* sm) {
+// 1 and ny - 1, ny in one thread each, for the Mur sides).  FINE: the fine
+// mesh over one coarse step; its coarse-fine sides take Eq. 5b from the lines
+// of levels n and n + 1 (interpolated in space once, blended in time per
+// sub-step), and the last sub-step's E goes to the coarse mesh (a8).
+template <class T, int C, int R, bool EDGE, bool FINE>
+__device__ __forceinline__ void multi_tile(const MultiArgs<T>& A, const FineArgs<T>* Fp, int bx, int by, int ox, int oy,
+                                           T* sm) {
   const MultiMesh<T>& M = A.C;
   const Mesh<T>& m = M.m;
   const Step<T>& c = M.c;
@@ -148,6 +177,8 @@ __device__ __forceinline__ void multi_tile(const MultiArgs<T>& A, int bx, int by
   const int ae = min(ax + A.tw, nx + 1), be = min(ay + A.th, ny + 1);   // owned [ax, ae) x [ay, be)
   T* rows = sm;                                    // [parity][warp][3][W]
   T* incs = sm + (size_t)2 * 3 * nw * W;           // [step][W]
+  const int Ht = R * nw;
+  T* lines = incs + (size_t)K * W;                 // FINE: bottom, top [W][2], left, right [Ht][2]
   // what no EM launch writes may be read before the previous launch is done:
   // the incident field's tables and the density
   for (int q = threadIdx.x; q < K * W; q += blockDim.x) {
@@ -180,6 +211,28 @@ __device__ __forceinline__ void multi_tile(const MultiArgs<T>& A, int bx, int by
     }
   }
   pdl_enter();
+  if constexpr (FINE && EDGE) {
+    const FineArgs<T>& F = *Fp;
+    for (int q = threadIdx.x; q < 2 * W + 2 * Ht; q += blockDim.x) {
+      const int sd = q < W ? SIDE_BOTTOM : q < 2 * W ? SIDE_TOP : q < 2 * W + Ht ? SIDE_LEFT : SIDE_RIGHT;
+      const bool hor = q < 2 * W;
+      const int e = q < W ? q : q < 2 * W ? q - W : q < 2 * W + Ht ? q - 2 * W : q - 2 * W - Ht;
+      const int smp = (hor ? ox : oy) + e;
+      const bool here = sd == SIDE_BOTTOM ? oy == 0 : sd == SIDE_TOP ? oy + Ht > ny : sd == SIDE_LEFT ? ox == 0 : ox + W > nx;
+      if (F.mode[sd] != BC_CFB || !here || smp >= (hor ? nx : ny)) continue;
+      // fine sample at coarse position start + (2 smp + 1 - r)/(2r), clamped (cfb_pos)
+      const int num = 2 * smp + 1 - F.r, den = 2 * F.r;
+      const int fl = num >= 0 ? num / den : -((-num + den - 1) / den);
+      int i = F.start[sd] + fl;
+      T xp = (T)(num - fl * den) / (T)den;
+      if (i < 0) { i = 0; xp = T(0); }
+      if (i > F.len[sd] - 2) { i = F.len[sd] - 2; xp = T(1); }
+      const T *o = F.old_line[sd], *l = F.new_line[sd];
+      const int st = F.stride[sd];
+      lines[2 * q] = o[i * st] * (T(1) - xp) + o[(i + 1) * st] * xp;
+      lines[2 * q + 1] = l[i * st] * (T(1) - xp) + l[(i + 1) * st] * xp;
+    }
+  }
   T ex[R][C], ey[R][C], hz[R][C], vx[R][C], vy[R][C], hzb[C];
   double s2[R][C];
 #pragma unroll
@@ -279,25 +332,42 @@ __device__ __forceinline__ void multi_tile(const MultiArgs<T>& A, int bx, int by
         ey[q][k] = mad_(cny[q][k], vy[q][k], mad_(-c.ce, hz[q][k] - hzl, ey[q][k]));
       }
       if constexpr (EDGE) {
-        // Mur left / right from the neighbouring column's old and new Ey
+        // sides left / right: Eq. 5b, or Mur from the neighbouring column's old and new Ey
+        const bool cl = FINE && Fp->mode[SIDE_LEFT] == BC_CFB, cr = FINE && Fp->mode[SIDE_RIGHT] == BC_CFB;
         const T orr = __shfl_down_sync(0xffffffffu, oy_[0], 1), nrr = __shfl_down_sync(0xffffffffu, ey[q][0], 1);
         const T oll = __shfl_up_sync(0xffffffffu, oy_[C - 1], 1), nll = __shfl_up_sync(0xffffffffu, ey[q][C - 1], 1);
-        if (i0 == 0)
+        if (i0 == 0 && !cl)
           ey[q][0] = C > 1 ? oy_[C - 1] + c.mur * (ey[q][C - 1] - oy_[0]) : orr + c.mur * (nrr - oy_[0]);
 #pragma unroll
         for (int k = 0; k < C; ++k)
-          if (i0 + k == nx)
+          if (i0 + k == nx && !cr)
             ey[q][k] = k > 0 ? oy_[0] + c.mur * (ey[q][0] - oy_[k]) : oll + c.mur * (nll - oy_[k]);
+        if constexpr (FINE) {
+          const T f = Fp->frac[s + 1];
+          const T* l = lines + 4 * W + 2 * (R * w + q);
+          if (i0 == 0 && cl) ey[q][0] = (T(1) - f) * l[0] + f * l[1];
+#pragma unroll
+          for (int k = 0; k < C; ++k)
+            if (i0 + k == nx && cr) ey[q][k] = (T(1) - f) * l[2 * Ht] + f * l[2 * Ht + 1];
+        }
       }
     }
     if constexpr (EDGE) {
       if (j0 == 0) {
+        const bool cb = FINE && Fp->mode[SIDE_BOTTOM] == BC_CFB;
+        const T f = FINE ? Fp->frac[s + 1] : T(0);
+        const T* l = lines + 2 * C * lane;
 #pragma unroll
-        for (int k = 0; k < C; ++k) ex[0][k] = b1[k] + c.mur * (ex[1][k] - b0[k]);
+        for (int k = 0; k < C; ++k)
+          ex[0][k] = cb ? (T(1) - f) * l[2 * k] + f * l[2 * k + 1] : b1[k] + c.mur * (ex[1][k] - b0[k]);
       }
       if (j0 + R - 1 == ny) {
+        const bool ct = FINE && Fp->mode[SIDE_TOP] == BC_CFB;
+        const T f = FINE ? Fp->frac[s + 1] : T(0);
+        const T* l = lines + 2 * W + 2 * C * lane;
 #pragma unroll
-        for (int k = 0; k < C; ++k) ex[R - 1][k] = t1[k] + c.mur * (ex[R - 2][k] - t0[k]);
+        for (int k = 0; k < C; ++k)
+          ex[R - 1][k] = ct ? (T(1) - f) * l[2 * k] + f * l[2 * k + 1] : t1[k] + c.mur * (ex[R - 2][k] - t0[k]);
       }
     }
     if (++lev == M.N) lev = 0;
@@ -335,11 +405,42 @@ __device__ __forceinline__ void multi_tile(const MultiArgs<T>& A, int bx, int by
       }
     }
   }
+  if constexpr (FINE) {
+    // a8: the means of r collinear fine edges, in the order of em_strips; the
+    // owned columns and rows start at multiples of r
+    const RestrW<T>& Wr = Fp->W;
+    if (!Wr.on) return;
+    __syncthreads();                               // the rows of the last sub-step have been read
+    T *sx = sm, *sy = sm + (size_t)W * Ht;
+#pragma unroll
+    for (int q = 0; q < R; ++q) {
+      TileVec<T, C>::st(sx + (R * w + q) * W + C * lane, ex[q]);
+      TileVec<T, C>::st(sy + (R * w + q) * W + C * lane, ey[q]);
+    }
+    __syncthreads();
+    const int r = Fp->r, hx = (ae - ax + r - 1) / r, hy = (be - ay + r - 1) / r;   // group heads
+    const unsigned mul = 0xffffffffu / (unsigned)hx + 1u;
+    for (int e = threadIdx.x; e < hx * hy; e += blockDim.x) {
+      const int gy = hx > 1 ? (int)__umulhi((unsigned)e, mul) : e, gx = e - gy * hx;
+      const int i = ax + r * gx, j = ay + r * gy, I = Wr.I0 + i / r, J = Wr.J0 + j / r;
+      const int at = (j - oy) * W + i - ox;
+      if (i < nx && J >= Wr.jlo && J <= Wr.jhi) {
+        T acc = sx[at];
+        for (int u = 1; u < r; ++u) acc = acc + sx[at + u];
+        Wr.cEx[J * Wr.cp + I] = acc * Wr.rinv;
+      }
+      if (j < ny && I >= Wr.ilo && I <= Wr.ihi) {
+        T acc = sy[at];
+        for (int u = 1; u < r; ++u) acc = acc + sy[at + u * W];
+        Wr.cEy[J * Wr.cp + I] = acc * Wr.rinv;
+      }
+    }
+  }
 }
 
 // block `t` of the tiles
-template <class T, int C, int R>
-__device__ __forceinline__ void multi_tiles(const MultiArgs<T>& A, int t, T* sm) {
+template <class T, int C, int R, bool FINE = false>
+__device__ __forceinline__ void multi_tiles(const MultiArgs<T>& A, int t, T* sm, const FineArgs<T>* Fp = nullptr) {
   const int by = t / A.gx, bx = t - by * A.gx;
   if (by >= A.gy) return;
   constexpr int W = 32 * C;
@@ -350,8 +451,8 @@ __device__ __forceinline__ void multi_tiles(const MultiArgs<T>& A, int t, T* sm)
   if (bx * A.tw >= A.z0 && min(bx * A.tw + A.tw, nx + 1) - 1 <= A.z2 && by * A.th >= A.z1 &&
       min(by * A.th + A.th, ny + 1) - 1 <= A.z3)
     return;                                          // all of it belongs to the near region
-  if (ox == 0 || ox + W > nx || oy == 0 || oy + H > ny) multi_tile<T, C, R, true>(A, bx, by, ox, oy, sm);
-  else multi_tile<T, C, R, false>(A, bx, by, ox, oy, sm);
+  if (ox == 0 || ox + W > nx || oy == 0 || oy + H > ny) multi_tile<T, C, R, true, FINE>(A, Fp, bx, by, ox, oy, sm);
+  else multi_tile<T, C, R, false, FINE>(A, Fp, bx, by, ox, oy, sm);
 }
 
 // ---------------------------------------------------------------------------
@@ -865,6 +966,12 @@ extern __shared__ __align__(16) char multi_smem[];
 template <class T, int C, int R, int TH>
 __global__ void __launch_bounds__(TH) k_multi(MultiArgs<T> A) {
   multi_tiles<T, C, R>(A, (int)blockIdx.x, reinterpret_cast<T*>(multi_smem));
+}
+
+// the r sub-steps of a fine mesh in one coarse step
+template <class T, int C, int R, int TH>
+__global__ void __launch_bounds__(TH) k_fine(MultiArgs<T> A, const __grid_constant__ FineArgs<T> F) {
+  multi_tiles<T, C, R, true>(A, (int)blockIdx.x, reinterpret_cast<T*>(multi_smem), &F);
 }
 
 // the near region: one cluster

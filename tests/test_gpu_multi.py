@@ -142,3 +142,29 @@ def test_batch_of_more_runs_than_one_launch_takes():
         for level in (0, 1):
             for f in FIELDS:
                 assert np.array_equal(batch.runs[q].read(f, level), one.read(f, level)), (q, f, level)
+
+
+@pytest.mark.parametrize("nx,ny,r,rect,kw", [
+    (120, 90, 3, (20, 11, 61, 44), {}), (120, 90, 4, (20, 11, 37, 28), {}), (120, 90, 4, (0, 0, 50, 33), {}),
+    (120, 90, 3, (70, 50, 120, 90), {}), (100, 90, 5, (3, 2, 16, 81), {}), (100, 90, 8, (30, 40, 38, 47), {}),
+    (100, 80, 4, (0, 7, 100, 70), dict(coupling=1)), (121, 97, 3, (30, 31, 75, 62), dict(boundary=1)),
+    (33, 20, 16, (4, 3, 9, 9), {}), (130, 70, 3, (10, 10, 32, 26), {})])
+def test_fine_sub_steps_in_one_launch(nx, ny, r, rect, kw):
+    """Fine meshes of a tile and more (64 columns): one column past a tile's,
+    ragged, at sides and corners, r that divides neither the columns nor the
+    rows of a tile, both couplings, CPML outside."""
+    a, b = _pair(nx, ny, r, rect, **kw)
+    _same(a, b, r, [1, 2, 13, 16, 5])
+
+
+@pytest.mark.parametrize("r", [2, 3])
+def test_fine_tiles_after_the_autotuner(r):
+    a, b = _pair(150, 140, r, (10, 20, 131, 122))
+    a.autotune()
+    a.set_graphs(True)
+    for n in (32, 64, 7):
+        a.advance(n)
+        b.advance(n)
+        for level in (0, 1):
+            for f in FIELDS:
+                assert np.array_equal(a.read(f, level), b.read(f, level)), (n, f, level)
