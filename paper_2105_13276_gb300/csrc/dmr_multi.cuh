@@ -61,19 +61,6 @@ __device__ __forceinline__ T node_sample(int i, int j, int nx, int ny, T exl, T 
   return sx + sy;
 }
 
-// v >= 0 (or NaN) as a double by integer operations: the conversion
-// instruction runs in the FP64 pipe, where the sum itself goes, and takes a
-// slot there even when predicated off.  The exponent is re-biased; a denormal
-// is scaled to a normal number first.
-__device__ __forceinline__ double to_f64(double v) { return v; }
-__device__ __forceinline__ double to_f64(float v) {
-  const unsigned b = __float_as_uint(v);
-  const bool den = b < 0x00800000u;
-  const unsigned x = den ? __float_as_uint(v * 16777216.f) : b;
-  const unsigned c = den ? 0x36800000u : (b >= 0x7f800000u ? 0x70000000u : 0x38000000u);
-  return __hiloint2double(x ? (int)((x >> 3) + c) : 0, (int)(x << 29));
-}
-
 // What the steps of one mesh share: the fields it starts from, where the new
 // level goes, the coefficients and the phase of the incident wave.
 template <class T>
@@ -317,8 +304,7 @@ __device__ __forceinline__ void multi_tile(const MultiArgs<T>& A, const FineArgs
           if constexpr (EDGE) {
             s2[q][k] += to_f64(node_sample(i0 + k, j0 + q, nx, ny, exl, ex[q][k], eyp, ey[q][k], inc[k]));
           } else {
-            const T sx = sq_mean(exl, ex[q][k]);
-            s2[q][k] += to_f64(sx + sq_mean(eyp + inc[k], ey[q][k] + inc[k]));
+            s2[q][k] = add_sample(s2[q][k], exl, ex[q][k], eyp + inc[k], ey[q][k] + inc[k]);
           }
         }
       }
@@ -597,8 +583,8 @@ __device__ __forceinline__ void near_step(T* sm, int ox, int oy, int wx, int wy,
     if (accum) {
       // at a side both edges of a pair are the one that is there
       // ((a^2 + a^2) / 2 = a^2 exactly)
-      const T sx = sq_mean(n.on_l ? ex[q] : exl, n.on_r ? exl : ex[q]);
-      n.s2[q] += to_f64(sx + sq_mean(eym + inc, (q == n.top ? eym : ey[q]) + inc));
+      n.s2[q] = add_sample(n.s2[q], n.on_l ? ex[q] : exl, n.on_r ? exl : ex[q], eym + inc,
+                           (q == n.top ? eym : ey[q]) + inc);
     }
     n.vx[q] = upd_v(c, n.vx[q], ex[q]);
     n.vy[q] = upd_v(c, n.vy[q], ey[q] + inc);
