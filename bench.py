@@ -44,7 +44,7 @@ FP64_INSTR_PEAK_T = 152 * 2.07e9 * 2 / 1e12
 # Ey + E_inc formed once; the E^2 sample 11), and the FP64 instructions the
 # kernels issue for them (each a * b + c one fused multiply-add)
 FP64_FLOPS_PER_NODE = (26.0, 37.0)
-FP64_INSTR_PER_NODE = (19.0, 28.0)
+FP64_INSTR_PER_NODE = (19.0, 26.0)
 
 
 def dist_env():
@@ -652,6 +652,10 @@ def run_ours(args):
                          "(60 B per node and step in FP32, 44 B on a period's first step, + the "
                          "coarse means) / the timed periods' total time (period-end kernels and "
                          "launch gaps included) / peak"}
+    if cfg.get("precision", 0) == 1 and cfg.get("boundary", 0) == 0:
+        roof["kernel_note"] = ("the one-step form; the timed periods advance several coarse steps per launch "
+                               "(k_multi, k_near) or all fine sub-steps of one (k_fine) where those are faster: "
+                               "frac_step is theirs, with bytes counted as if every step streamed the state")
     if len(forms0) > 2:
         roof["fine_substep"] = form_roof(2)
         roof["fine_substep"]["kernel"] = ("k_em_w2 (two node columns per lane)" if shape[2] == 2
@@ -679,7 +683,7 @@ def run_ours(args):
                 "avg_launch_us": a_mid["avg_launch_us"],
                 "fp64_flops_per_launch": a_mid["fp64_flops_per_launch"],
                 "fp64_pipe": a_mid["fp64_pipe"],
-                "ops_note": "37 FP64 flops per node with the E^2 sample, 26 without, issued as 28 / "
+                "ops_note": "37 FP64 flops per node with the E^2 sample, 26 without, issued as 26 / "
                             "19 FP64 instructions (fused multiply-adds); fp64_pipe: those "
                             "instructions against 2 per clock per SM; nodes from the launch's "
                             "algorithmic bytes (11 words per node, + 16 B of the E^2 sum)",
