@@ -2040,14 +2040,67 @@ struct Engine final : Base {
     return s_;
   }
 
+  // While a segment is recomputed, E and v of both meshes live on the tape: a
+  // step reads the slots that the step before it wrote and writes slots of its
+  // own, so the records are pointers and nothing is copied (a gather of 12
+  // arrays per coarse step before, bound by the copy: 512^2, r = 2, backward of
+  // 512 steps in one segment 29.2 ms then, 27.1 ms now).
+  // Only what still lies in the workspace (a segment's first step, the fine mesh
+  // after growth) is copied.  The buffer tables point at the slots meanwhile.
+  struct Buffers {
+    T *c[2][5], *f0[2][6], *f1[2][5];
+  };
+  Buffers save_buffers() const {
+    Buffers B;
+    memcpy(B.c, cE, sizeof cE);
+    memcpy(B.f0, fptr, sizeof fptr);
+    memcpy(B.f1, fE1, sizeof fE1);
+    return B;
+  }
+  void load_fine_buffers(const Buffers& B, int set) {
+    memcpy(fptr[set], B.f0[set], sizeof fptr[set]);
+    memcpy(fE1[set], B.f1[set], sizeof fE1[set]);
+  }
+  // The workspace's own buffers again, with the present E and v in them.  Edges
+  // only: what lies between a row's last edge and the next row is 0 in the
+  // workspace and undefined on the tape, where no kernel writes or reads it.
+  int leave_tape(const Buffers& B) {
+    int s = DMR_OK;
+    auto put = [&](T* to, const T* from, int q, int nx, int ny, int p) {
+      const bool x = q == 0 || q == 3;               // Ex, vx: nx x (ny + 1) edges
+      if (!s && to != from)
+        s = ck(cudaMemcpy2DAsync(to, (size_t)p * L.es, from, (size_t)p * L.es, (size_t)(x ? nx : nx + 1) * L.es,
+                                 x ? ny + 1 : ny, cudaMemcpyDeviceToDevice, st), "leave tape");
+    };
+    for (int q : {0, 1, 3, 4}) {
+      put(B.c[cpar][q], cE[cpar][q], q, C.nx, C.ny, C.p);
+      if (has_fine)
+        put(fpar ? B.f1[cur][q] : B.f0[cur][q], fineE(cur, fpar, q), q, F[cur].nx, F[cur].ny, F[cur].p);
+    }
+    memcpy(cE, B.c, sizeof cE);
+    for (int set = 0; set < 2; ++set) load_fine_buffers(B, set);
+    C.Ex = cE[cpar][0]; C.Ey = cE[cpar][1]; C.Hz = cE[cpar][2]; C.vx = cE[cpar][3]; C.vy = cE[cpar][4];
+    if (has_fine) {
+      F[cur].Ex = fineE(cur, fpar, 0); F[cur].Ey = fineE(cur, fpar, 1); F[cur].Hz = fineE(cur, fpar, 2);
+      F[cur].vx = fineE(cur, fpar, 3); F[cur].vy = fineE(cur, fpar, 4);
+    }
+    return s;
+  }
+  // a record of array p: itself if it is on the tape, a copy otherwise
+  const T* tape_keep(const T* p, size_t bytes) {
+    const char* c = reinterpret_cast<const char*>(p);
+    return c >= tape && c < tape + tape_cap ? p : tape_copy(p, bytes);
+  }
+  // slots for a launch's E and v outputs
+  bool tape_outputs(T** ex, T** ey, T** vx, T** vy, size_t bytes) {
+    T** const o[4] = {ex, ey, vx, vy};
+    for (T** q : o)
+      if (!(*q = reinterpret_cast<T*>(tape_slot(bytes)))) return false;
+    return true;
+  }
+
   // one coarse step with its tape records: the launches of launch_coarse_step
-  // (the coarse step with the first fine sub-step, then sub-steps 2..r) with
-  // the tape copies queued after each and flushed before any launch that
-  // overwrites their sources (double buffering keeps the inputs of a launch
-  // until the launch after it).  At r = 2 one flush per coarse step, before
-  // its first launch, covers all of them: the step's own inputs are queued
-  // ahead of it, and what the step leaves (v outputs, sub-step 2's inputs)
-  // stays intact until the next step's first launch.
+  // (the coarse step with the first fine sub-step, then sub-steps 2..r)
   int record_step(StepRec* R) {
     const int r = cfg.r;
     R->m = m;
@@ -2055,59 +2108,53 @@ struct Engine final : Base {
     R->fine = has_fine;
     R->rvalid = rvalid;
     const int cp0 = cpar;
-    const bool one_flush = has_fine && r == 2;
     const size_t fb = has_fine ? fplane_b(rect) : 0;
-    if (one_flush) {
-      R->cEx = tape_copy(C.Ex, cplane_b());          // E^n
-      R->cEy = tape_copy(C.Ey, cplane_b());
-      R->fEx.push_back(tape_copy(F[cur].Ex, fb));    // sub-step 1's input
-      R->fEy.push_back(tape_copy(F[cur].Ey, fb));
-      flush_tape();
-    }
+    auto fine_slots = [&]() {
+      T** const t = fpar ? fptr[cur] : fE1[cur];     // the buffers of the other parity
+      R->fEx.push_back(tape_keep(F[cur].Ex, fb));    // the sub-step's input
+      R->fEy.push_back(tape_keep(F[cur].Ey, fb));
+      return tape_outputs(t + 0, t + 1, t + 3, t + 4, fb);
+    };
+    R->cEx = tape_keep(C.Ex, cplane_b());            // E^n
+    R->cEy = tape_keep(C.Ey, cplane_b());
+    bool ok = tape_outputs(&cE[cpar ^ 1][0], &cE[cpar ^ 1][1], &cE[cpar ^ 1][3], &cE[cpar ^ 1][4], cplane_b());
+    if (ok && has_fine) ok = fine_slots();
+    if (!ok) return fail(DMR_ECAPACITY, "adjoint tape overflow");
+    flush_tape();
     dmr::EmArgs<T> Ac, Af;
     em_args_for(1, m, cpar, fpar, rvalid, &Ac, has_fine ? &Af : nullptr);
     if (has_fine) go_em2(Ac.nblk + Ac.ncfb + Af.nblk + Af.ncfb, Ac, Af);
     else go_em(Ac.nblk + Ac.ncfb, Ac);
     counted(1);
-    if (!one_flush) {
-      R->cEx = tape_copy(C.Ex, cplane_b());        // E^n (this step's input parity)
-      R->cEy = tape_copy(C.Ey, cplane_b());
-    }
     flip_coarse();
-    R->cvx = tape_copy(C.vx, cplane_b());        // v^{n+1/2}
-    R->cvy = tape_copy(C.vy, cplane_b());
+    R->cvx = C.vx;                                   // v^{n+1/2}
+    R->cvy = C.vy;
     if (has_fine) {
       for (int k = 1; k <= r; ++k) {
         if (k > 1) {
+          if (!fine_slots()) return fail(DMR_ECAPACITY, "adjoint tape overflow");
           em_args_for(k, m, cp0, fpar, rvalid, nullptr, &Af);
           go_em(Af.nblk + Af.ncfb, Af);
           counted(1);
         }
-        if (!(one_flush && k == 1)) {
-          R->fEx.push_back(tape_copy(F[cur].Ex, fb));   // the sub-step's input
-          R->fEy.push_back(tape_copy(F[cur].Ey, fb));
-        }
         flip_fine();
-        R->fvx.push_back(tape_copy(F[cur].vx, fb));   // its v output
-        R->fvy.push_back(tape_copy(F[cur].vy, fb));
-        if (!one_flush) flush_tape();
+        R->fvx.push_back(F[cur].vx);                 // its v output
+        R->fvy.push_back(F[cur].vy);
       }
       rvalid = true;
-    } else {
-      flush_tape();
     }
     ++m;
     return launched("recorded EM step");
   }
 
-  int record_period(PerRec* P) {
+  int record_period(PerRec* P, const Buffers& own) {
     P->L = m;
     for (int k = 0; k < 4; ++k) P->rect_b[k] = rect[k];
     P->cur_b = cur;
     P->fine = has_fine;
     P->rvalid = rvalid;
-    P->cEx = tape_copy(C.Ex, cplane_b());
-    P->cEy = tape_copy(C.Ey, cplane_b());
+    P->cEx = tape_keep(C.Ex, cplane_b());
+    P->cEy = tape_keep(C.Ey, cplane_b());
     P->nc = tape_copy(C.n, cplane_b());
     double* s2c = tape_alloc_d(L.cplane * 8);
     if (s2c)
@@ -2115,8 +2162,8 @@ struct Engine final : Base {
     P->S2c = s2c;
     if (has_fine) {
       const size_t fb = fplane_b(rect);
-      P->fEx = tape_copy(F[cur].Ex, fb);
-      P->fEy = tape_copy(F[cur].Ey, fb);
+      P->fEx = tape_keep(F[cur].Ex, fb);
+      P->fEy = tape_keep(F[cur].Ey, fb);
       P->nf = tape_copy(F[cur].n, fb);
       double* s2f = tape_alloc_d(fb / L.es * 8);
       if (s2f)
@@ -2125,6 +2172,7 @@ struct Engine final : Base {
       P->S2f = s2f;
     }
     flush_tape();   // before the period end rewrites n
+    load_fine_buffers(own, cur ^ 1);   // growth fills the other fine set in the workspace
     if (int s = launch_period_end(m)) return s;
     if (int s = period_end_host()) return s;
     P->expanded = has_fine && (rect[0] != P->rect_b[0] || rect[1] != P->rect_b[1] ||
@@ -2249,6 +2297,7 @@ struct Engine final : Base {
     if (!st_) st_ = ck(cudaStreamWaitEvent(sq, ev_go, 0), "stream wait");
     std::vector<StepRec> steps[2];
     std::vector<PerRec> pers[2];
+    const Buffers own = save_buffers();
     // restore segment sg's start and recompute it onto tape sg & 1, on sq
     auto recompute = [&](int sg) -> int {
       const int b = sg & 1;
@@ -2257,6 +2306,8 @@ struct Engine final : Base {
       tape_cap = tseg;
       tape_used = 0;
       tape_over = false;
+      tjobs.n = 0;
+      tjob_max16 = 0;
       int s_ = ck(cudaMemcpyAsync(ws, rec.ckpt + (size_t)sg * wbytes(), L.total, cudaMemcpyDeviceToDevice, st),
                   "restore checkpoint");
       if (!s_) {
@@ -2274,8 +2325,10 @@ struct Engine final : Base {
           }
           if (s_) break;
           pers[b].emplace_back();
-          s_ = record_period(&pers[b].back());
+          s_ = record_period(&pers[b].back(), own);
         }
+        const int l_ = leave_tape(own);
+        if (!s_) s_ = l_;
       }
       if (!s_ && tape_over) s_ = fail(DMR_ECAPACITY, "adjoint tape overflow");
       if (!s_) s_ = ck(cudaEventRecord(ev_rec[b], sq), "event record");
