@@ -1462,7 +1462,13 @@ struct Engine final : Base {
     A.C.w = dmr::Wts{cfg.nx, cfg.ny, has_fine ? 1 : 0, rect[0], rect[1], rect[2], rect[3]};
     A.C.D = c_D; A.C.nu = c_nu; A.C.ntmp = c_ntmp; A.C.erms = cErms;
     A.C.partP = part[0]; A.C.partN = part[2];
-    A.C.gx = (int)gc.x; A.C.nb = (int)(gc.x * gc.y);
+    // several rows per thread from a few blocks per SM on
+    auto tiles = [&](dmr::PeMesh<T>& M, const dim3& g) {
+      M.u = (int)(g.x * g.y) >= 16 * num_sms ? dmr::kPeRows : 1;
+      M.gx = (int)g.x;
+      M.nb = (int)(g.x * ((g.y + M.u - 1) / M.u));
+    };
+    tiles(A.C, gc);
     A.F.nb = 0;
     A.F.partP = part[1]; A.F.partN = part[3];
     A.r = r;
@@ -1482,7 +1488,7 @@ struct Engine final : Base {
       A.F.d = make_dens(r);
       A.F.w = dmr::Wts{f.nx, f.ny, 0, 0, 0, 0, 0};
       A.F.D = f_D; A.F.nu = f_nu; A.F.ntmp = f_ntmp; A.F.erms = fErms[cur];
-      A.F.gx = (int)gf.x; A.F.nb = (int)(gf.x * gf.y);
+      tiles(A.F, gf);
       dmr::Dir<T>& dir = A.dir;
       dir.r = r;
       for (int q = 0; q < 4; ++q) {

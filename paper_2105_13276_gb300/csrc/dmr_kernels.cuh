@@ -127,6 +127,13 @@ __device__ __forceinline__ double to_f64(float v) {
   return __hiloint2double(x ? (int)((x >> 3) + c) : 0, (int)(x << 29));
 }
 
+// any float as a double, as to_f64
+__device__ __forceinline__ double to_f64_any(double v) { return v; }
+__device__ __forceinline__ double to_f64_any(float v) {
+  const double d = to_f64(fabsf(v));
+  return __hiloint2double(__double2hiint(d) | (int)(__float_as_uint(v) & 0x80000000u), __double2loint(d));
+}
+
 // s2 + (a^2 + b^2)/2 + (e^2 + f^2)/2, the E^2 sample of a node with two edges
 // each way: the halves are exact, so one factor 1/2 in the sum's fused
 // multiply-add gives the bits of halving each mean first, and costs two
@@ -1285,6 +1292,12 @@ __device__ __forceinline__ double trap_w(const Wts& w, int i, int j) {
   return v;
 }
 
+// whether the weight is 1 (nodes away from the mesh's and the rectangle's sides)
+__device__ __forceinline__ bool trap_one(const Wts& w, int i, int j) {
+  return i > 0 && i < w.nx && j > 0 && j < w.ny &&
+         !(w.has_rect && i >= w.I0 && i <= w.I1 && j >= w.J0 && j <= w.J1);
+}
+
 // deterministic block sum of a double (blockDim.x*blockDim.y threads, <= 1024)
 __device__ __forceinline__ double block_sum(double v) {
   __shared__ double sh[32];
@@ -1321,8 +1334,15 @@ struct PeMesh {
   Wts w;
   T *D, *nu, *ntmp, *erms;
   double *partP, *partN;
-  int gx, nb;
+  int gx, nb, u;       // u: node rows per thread (1 or kPeRows)
 };
+// Node rows per thread of the period-end launches on a larger mesh: a thread
+// adds its rows' terms before the block's sum, which costs five FP64 adds per
+// warp and row (16 cycles of the SM's FP64 pipe each); a smaller mesh keeps one
+// row per thread, for the blocks.  FP32, all steps of a period with its end:
+// uniform 1024^2 861 to 840 us, 2048 x 1024 with a quarter refined r = 2 4.24 to
+// 4.12 ms, r = 4 14.02 to 13.72 ms, a batch of 16 runs 8.90 to 8.47 ms.
+constexpr int kPeRows = 4;
 
 // Dirichlet (coarse-fine) sides of the fine density step: new coarse density
 // interpolated along the side (Eq. 5b, frac = 1).
@@ -1352,12 +1372,12 @@ struct PeArgs {
   int nsched;
 };
 
-// node (i, j) of mesh-block b of a PeMesh (false past the mesh)
+// node (i, j) of row u of the thread in mesh-block b of a PeMesh (false past the mesh)
 template <class T>
-__device__ __forceinline__ bool pe_node(const PeMesh<T>& M, int b, int* i, int* j) {
+__device__ __forceinline__ bool pe_node(const PeMesh<T>& M, int b, int u, int* i, int* j) {
   const int by = b / M.gx, bx = b - by * M.gx;
   *i = bx * TX + (int)threadIdx.x;
-  *j = by * TY + (int)threadIdx.y;
+  *j = (by * M.u + u) * TY + (int)threadIdx.y;
   return *i <= M.m.nx && *j <= M.m.ny;
 }
 
@@ -1370,8 +1390,9 @@ __device__ __forceinline__ double rates_node(const PeMesh<T>& M, int i, int j) {
   const Mesh<T>& m = M.m;
   const Dens& d = M.d;
   const int id = j * m.p + i;
-  const double s2 = m.S2[id] + (double)node_e2(m, M.c, i, j);
-  const double e2 = eeff2_of(s2, d);
+  const double s2 = m.S2[id] + to_f64(node_e2(m, M.c, i, j));
+  const double ms = s2 * d.invN;
+  const double e2 = ms * d.invg;     // eeff2_of(s2, d)
   const T nui = nu_ion<T>(e2, d);
   T n = m.n[id];
   T wp2 = n * (T)d.wp2c;
@@ -1379,9 +1400,10 @@ __device__ __forceinline__ double rates_node(const PeMesh<T>& M, int i, int j) {
   T den = nui * (T)d.nu_m + wp2;
   M.D[id] = (den == T(0)) ? (T)d.De : num / den;
   M.nu[id] = nui - (T)d.nu_a;
-  M.erms[id] = sqrt((T)(s2 * d.invN));
+  M.erms[id] = sqrt((T)ms);
   m.S2[id] = 0.0;
-  return trap_w(M.w, i, j) * (double)n * d.heat * e2;
+  const double dn = to_f64_any(n);
+  return (trap_one(M.w, i, j) ? dn : trap_w(M.w, i, j) * dn) * d.heat * e2;
 }
 
 // a9 second pass at node (i, j): forward-Euler continuity step over one
@@ -1437,9 +1459,12 @@ __global__ void __launch_bounds__(TX * TY) k_pe_rates(PeArgs<T> A) {
   const bool fine = b >= A.C.nb;
   const PeMesh<T>& M = fine ? A.F : A.C;
   const int mb = fine ? b - A.C.nb : b;
-  int i, j;
   double contrib = 0.0;
-  if (pe_node(M, mb, &i, &j)) contrib = rates_node(M, i, j);
+#pragma unroll 2
+  for (int u = 0; u < M.u; ++u) {
+    int i, j;
+    if (pe_node(M, mb, u, &i, &j)) contrib += rates_node(M, i, j);
+  }
   const double s = block_sum(contrib);
   if (threadIdx.x == 0 && threadIdx.y == 0) M.partP[mb] = s;
 }
@@ -1451,17 +1476,22 @@ __global__ void __launch_bounds__(TX * TY) k_pe_density(PeArgs<T> A) {
   const int b = (int)blockIdx.x;
   const bool fine = b >= A.C.nb;
   const PeMesh<T>& M = fine ? A.F : A.C;
-  int i, j;
-  if (!pe_node(M, fine ? b - A.C.nb : b, &i, &j)) return;
-  const int id = j * M.m.p + i;
-  if (fine) {
-    const Dir<T>& d = A.dir;
-    if (d.on[SIDE_BOTTOM] && j == 0) { M.ntmp[id] = dir_value(d, A.C, SIDE_BOTTOM, i); return; }
-    if (d.on[SIDE_TOP] && j == M.m.ny) { M.ntmp[id] = dir_value(d, A.C, SIDE_TOP, i); return; }
-    if (d.on[SIDE_LEFT] && i == 0) { M.ntmp[id] = dir_value(d, A.C, SIDE_LEFT, j); return; }
-    if (d.on[SIDE_RIGHT] && i == M.m.nx) { M.ntmp[id] = dir_value(d, A.C, SIDE_RIGHT, j); return; }
+#pragma unroll 2
+  for (int u = 0; u < M.u; ++u) {
+    int i, j;
+    if (!pe_node(M, fine ? b - A.C.nb : b, u, &i, &j)) return;   // the later rows are past the mesh too
+    const int id = j * M.m.p + i;
+    if (fine) {
+      const Dir<T>& d = A.dir;
+      int sd = -1, q = 0;
+      if (d.on[SIDE_RIGHT] && i == M.m.nx) { sd = SIDE_RIGHT; q = j; }
+      if (d.on[SIDE_LEFT] && i == 0) { sd = SIDE_LEFT; q = j; }
+      if (d.on[SIDE_TOP] && j == M.m.ny) { sd = SIDE_TOP; q = i; }
+      if (d.on[SIDE_BOTTOM] && j == 0) { sd = SIDE_BOTTOM; q = i; }
+      if (sd >= 0) { M.ntmp[id] = dir_value(d, A.C, sd, q); continue; }
+    }
+    M.ntmp[id] = density_new(M, i, j);
   }
-  M.ntmp[id] = density_new(M, i, j);
 }
 
 // the new coarse density at node (i, j) as the commit writes it: the fine
@@ -1579,16 +1609,19 @@ __global__ void __launch_bounds__(TX * TY) k_pe_commit(PeArgs<T> A) {
   if (flagged && threadIdx.x == 0 && threadIdx.y == 0)
     flags = FlagSum{0ull, {0x7fffffff, 0x7fffffff, -1, -1}, 0, 0, 0};
   __syncthreads();
-  int i, j;
   double contrib = 0.0;
-  const bool in = pe_node(M, mb, &i, &j);
-  T v = T(0);
-  if (in) {
-    v = fine ? M.ntmp[j * M.m.p + i] : committed_coarse(A, i, j);
-    M.m.n[j * M.m.p + i] = v;
-    contrib = trap_w(M.w, i, j) * (double)v;
+  for (int u = 0; u < M.u; ++u) {
+    int i, j;
+    const bool in = pe_node(M, mb, u, &i, &j);
+    T v = T(0);
+    if (in) {
+      v = fine ? M.ntmp[j * M.m.p + i] : committed_coarse(A, i, j);
+      M.m.n[j * M.m.p + i] = v;
+      const double dv = to_f64_any(v);
+      contrib += trap_one(M.w, i, j) ? dv : trap_w(M.w, i, j) * dv;
+    }
+    if (flagged) flag_node(A, in, i, j, v, &flags);
   }
-  if (flagged) flag_node(A, in, i, j, v, &flags);
   const double s = block_sum(contrib);          // its barriers order the flags' sums too
   if (threadIdx.x == 0 && threadIdx.y == 0) {
     if (flagged) flag_commit(A.ctl, flags);
