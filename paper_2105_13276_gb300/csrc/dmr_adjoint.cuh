@@ -59,37 +59,6 @@ struct FwdM {                 // recorded forward values of the step
 
 struct Modes { int m[4]; };
 
-template <class T>
-__device__ __forceinline__ T adj_x(const AdjM<T>& a, const Modes& md, T mur, int i, int j) {
-  // adjoint of interior E'_x(i,j) including what the Mur rows took from it
-  const int p = a.p;
-  T v = a.aEx_in[j * p + i];
-  if (j == 1 && md.m[SIDE_BOTTOM] == BC_MUR) v = v + mur * a.aEx_in[i];
-  if (j == a.ny - 1 && md.m[SIDE_TOP] == BC_MUR) v = v + mur * a.aEx_in[a.ny * p + i];
-  return v;
-}
-
-template <class T>
-__device__ __forceinline__ T adj_y(const AdjM<T>& a, const Modes& md, T mur, int i, int j) {
-  const int p = a.p;
-  T v = a.aEy_in[j * p + i];
-  if (i == 1 && md.m[SIDE_LEFT] == BC_MUR) v = v + mur * a.aEy_in[j * p];
-  if (i == a.nx - 1 && md.m[SIDE_RIGHT] == BC_MUR) v = v + mur * a.aEy_in[j * p + a.nx];
-  return v;
-}
-
-// The adjoint of H^{l-1/2} at cell (i, j): that of H^{l+1/2} plus
-// ce curlH^T(aE') over the interior edges (after the Mur rows' share).
-template <class T>
-__device__ __forceinline__ T ka_h_value(const AdjM<T>& a, const Step<T>& c, const Modes& md, int i, int j) {
-  T acc = T(0);
-  if (j > 0) acc = acc + adj_x(a, md, c.mur, i, j);
-  if (j + 1 < a.ny) acc = acc - adj_x(a, md, c.mur, i, j + 1);
-  if (i > 0) acc = acc - adj_y(a, md, c.mur, i, j);
-  if (i + 1 < a.nx) acc = acc + adj_y(a, md, c.mur, i + 1, j);
-  return a.aHz[j * a.p + i] + c.ce * acc;
-}
-
 __device__ __forceinline__ double block_sum_d(double v) { return block_sum(v); }
 
 // Coarse side of a reversed coarse step (nullptrs / off on a fine mesh or
@@ -115,130 +84,154 @@ struct CoarseT {
 // edges of the node need), then the gather of aE^l (edges (i, j)), av, an;
 // returns the node's E0 share.  The edge adjoints of E^l are stored (the
 // output buffer is not cleared before); with a CoarseT the side shares are
-// added and a8 transposed.  Every load of a thread comes before its first
-// store, so the loads of the in-place arrays (av, an, side lines) and of the
-// read-only inputs are all in flight at once.
+// added and a8 transposed.
+// Bound by latency: a reversed coarse step is a chain of r + 1 launches of few
+// blocks each.  So all loads come first and none is behind a branch that
+// differs within a block: absent edges count 0, the Mur rows' shares are
+// selects, and 64 registers hold what is in flight.  (With the loads where the
+// formulas need them, behind the edge tests, the compiler kept 32 registers and
+// a thread made one trip to L2 after the other: 13.9 us per launch cold, of 12
+// blocks as of 580.)  512^2, r = 2, 512 steps recorded and reversed, FP32: 27.8
+// to 23.1 ms; 40 x 32 in FP64, 128 steps: 10.7 to 9.5 ms.
 template <class T>
 __device__ __forceinline__ T ka_e_node(const AdjM<T>& a, const FwdM<T>& f, const Step<T>& c, const Modes& md,
                                        const CoarseT<T>& ct, int i, int j) {
   const int nx = a.nx, ny = a.ny, p = a.p;
-  T e0 = T(0);
-  if (i <= nx && j <= ny) {
-    const int id = j * p + i;
-    const bool xe = i < nx, ye = j < ny;
-    // ---- H adjoints of the cells the node's edges border
-    const T h00 = (xe && ye) ? ka_h_value(a, c, md, i, j) : T(0);
-    const T h0m = (xe && j > 0) ? ka_h_value(a, c, md, i, j - 1) : T(0);
-    const T hm0 = (ye && i > 0) ? ka_h_value(a, c, md, i - 1, j) : T(0);
-    // ---- loads: in-place values and side lines
-    const T avx0 = xe ? a.avx[id] : T(0);
-    const T avy0 = ye ? a.avy[id] : T(0);
-    const T an0 = a.an[id];
-    const bool s_b = xe && ct.side_on[SIDE_BOTTOM] && j == ct.side_at[SIDE_BOTTOM];
-    const bool s_t = xe && ct.side_on[SIDE_TOP] && j == ct.side_at[SIDE_TOP];
-    const bool s_l = ye && ct.side_on[SIDE_LEFT] && i == ct.side_at[SIDE_LEFT];
-    const bool s_r = ye && ct.side_on[SIDE_RIGHT] && i == ct.side_at[SIDE_RIGHT];
-    const T v_b = s_b ? ct.side[SIDE_BOTTOM][i] : T(0);
-    const T v_t = s_t ? ct.side[SIDE_TOP][i] : T(0);
-    const T v_l = s_l ? ct.side[SIDE_LEFT][j] : T(0);
-    const T v_r = s_r ? ct.side[SIDE_RIGHT][j] : T(0);
-    T an_acc = T(0);
-    // ---- x edge (i, j)
-    T outx = T(0), avx1 = T(0);
-    if (xe) {
-      T out, avt;
-      if (j > 0 && j < ny) {
-        const T aEa = adj_x(a, md, c.mur, i, j);
-        avt = avx0 + c.cj * (f.n[id] + f.n[id + 1]) * aEa;
-        out = aEa;
-        if (j == 1 && md.m[SIDE_BOTTOM] == BC_MUR) out = out + a.aEx_in[i];
-        if (j == ny - 1 && md.m[SIDE_TOP] == BC_MUR) out = out + a.aEx_in[ny * p + i];
-        an_acc = an_acc + f.vx[id] * aEa;
-      } else {
-        const int sd = j == 0 ? SIDE_BOTTOM : SIDE_TOP;
-        avt = avx0;
-        out = md.m[sd] == BC_MUR ? -c.mur * a.aEx_in[id] : T(0);
-      }
-      out = out - c.vb * avt;
-      T hs = T(0);
-      if (j < ny) hs = hs + h00;
-      if (j > 0) hs = hs - h0m;
-      out = out - c.ch * hs;
-      if (c.accum) {
-        const T wl = (i > 0) ? T(0.5) : T(1);                 // node i: this is its right edge
-        const T wr = (i + 1 < nx) ? T(0.5) : T(1);            // node i+1: its left edge
-        out = out + T(2) * f.Ex[id] * (a.aS2[id] * wl + a.aS2[id + 1] * wr);
-      }
-      avx1 = c.va * avt;
-      if (s_b) out = v_b + out;
-      if (s_t) out = v_t + out;
-      outx = out;
+  if (i > nx || j > ny) return T(0);
+  const int id = j * p + i;
+  const bool xe = i < nx, ye = j < ny;
+  auto ld = [](const T* q, bool v) { return v ? *q : T(0); };
+  // edges whose E' the interior formula gives: 0 < j < ny (x), 0 < i < nx (y)
+  const bool jin = j > 0 && j < ny, iin = i > 0 && i < nx;
+  const bool jdn = j > 1, jup = j + 1 < ny, ilf = i > 1, irt = i + 1 < nx;   // the same one row / column on
+  T x00 = ld(a.aEx_in + id, xe && jin);
+  T x0p = ld(a.aEx_in + id + p, xe && jup);
+  T x0m = ld(a.aEx_in + id - p, xe && jdn);
+  T xm0 = ld(a.aEx_in + id - 1, i > 0 && jin);
+  T xmp = ld(a.aEx_in + id + p - 1, i > 0 && jup);
+  T y00 = ld(a.aEy_in + id, ye && iin);
+  T yp0 = ld(a.aEy_in + id + 1, ye && irt);
+  T ym0 = ld(a.aEy_in + id - 1, ye && ilf);
+  T y0m = ld(a.aEy_in + id - p, j > 0 && iin);
+  T ypm = ld(a.aEy_in + id - p + 1, j > 0 && irt);
+  const T hz00 = ld(a.aHz + id, xe && ye);
+  const T hz0m = ld(a.aHz + id - p, xe && j > 0);
+  const T hzm0 = ld(a.aHz + id - 1, ye && i > 0);
+  const T avx0 = ld(a.avx + id, xe), avy0 = ld(a.avy + id, ye), an0 = a.an[id];
+  const T n00 = f.n[id], np0 = ld(f.n + id + 1, xe), n0p = ld(f.n + id + p, ye);
+  const T vx0 = ld(f.vx + id, xe && jin), vxm = ld(f.vx + id - 1, i > 0 && jin);
+  const T vy0 = ld(f.vy + id, ye && iin), vym = ld(f.vy + id - p, j > 0 && iin);
+  const T ckx = c.ckx[i], skx = c.skx[i];
+  const T ex = ld(f.Ex + id, c.accum && xe), ey0 = ld(f.Ey + id, c.accum && ye);
+  const T s00 = ld(a.aS2 + id, c.accum), sp0 = ld(a.aS2 + id + 1, c.accum && xe), s0p = ld(a.aS2 + id + p, c.accum && ye);
+  const bool s_b = xe && ct.side_on[SIDE_BOTTOM] && j == ct.side_at[SIDE_BOTTOM];
+  const bool s_t = xe && ct.side_on[SIDE_TOP] && j == ct.side_at[SIDE_TOP];
+  const bool s_l = ye && ct.side_on[SIDE_LEFT] && i == ct.side_at[SIDE_LEFT];
+  const bool s_r = ye && ct.side_on[SIDE_RIGHT] && i == ct.side_at[SIDE_RIGHT];
+  const T v_b = ld(ct.side[SIDE_BOTTOM] + i, s_b), v_t = ld(ct.side[SIDE_TOP] + i, s_t);
+  const T v_l = ld(ct.side[SIDE_LEFT] + j, s_l), v_r = ld(ct.side[SIDE_RIGHT] + j, s_r);
+  // ---- Mur sides: row 1 of Ex gave mur E' to row 0 (and so on), so its adjoint
+  // takes mur times row 0's; bx0, bxm: row 0 or ny of columns i, i - 1, by0, bym:
+  // column 0 or nx of rows j, j - 1
+  const bool mb = md.m[SIDE_BOTTOM] == BC_MUR && j <= 2, mt = md.m[SIDE_TOP] == BC_MUR && j >= ny - 2;
+  const bool ml = md.m[SIDE_LEFT] == BC_MUR && i <= 2, mr = md.m[SIDE_RIGHT] == BC_MUR && i >= nx - 2;
+  const T b0 = ld(a.aEx_in + i, mb && xe), bm = ld(a.aEx_in + i - 1, mb && i > 0);
+  const T t0 = ld(a.aEx_in + ny * p + i, mt && xe), tm = ld(a.aEx_in + ny * p + i - 1, mt && i > 0);
+  const T l0 = ld(a.aEy_in + j * p, ml && ye), lm = ld(a.aEy_in + (j - 1) * p, ml && j > 0);
+  const T r0 = ld(a.aEy_in + j * p + nx, mr && ye), rm = ld(a.aEy_in + (j - 1) * p + nx, mr && j > 0);
+  auto mur = [&](T v, bool on, T w) { return on ? v + c.mur * w : v; };
+  x00 = mur(mur(x00, mb && j == 1, b0), mt && j == ny - 1, t0);
+  x0p = mur(mur(x0p, mb && j == 0, b0), mt && j == ny - 2, t0);
+  x0m = mur(mur(x0m, mb && j == 2, b0), mt && j == ny, t0);
+  xm0 = mur(mur(xm0, mb && j == 1, bm), mt && j == ny - 1, tm);
+  xmp = mur(mur(xmp, mb && j == 0, bm), mt && j == ny - 2, tm);
+  y00 = mur(mur(y00, ml && i == 1, l0), mr && i == nx - 1, r0);
+  yp0 = mur(mur(yp0, ml && i == 0, l0), mr && i == nx - 2, r0);
+  ym0 = mur(mur(ym0, ml && i == 2, l0), mr && i == nx, r0);
+  y0m = mur(mur(y0m, ml && i == 1, lm), mr && i == nx - 1, rm);
+  ypm = mur(mur(ypm, ml && i == 0, lm), mr && i == nx - 2, rm);
+  // ---- adjoint of H^{l-1/2} at the cells (i, j), (i, j - 1), (i - 1, j): that
+  // of H^{l+1/2} plus ce curlH^T(aE') over the interior edges
+  const T h00 = (xe && ye) ? hz00 + c.ce * (x00 - x0p - y00 + yp0) : T(0);
+  const T h0m = (xe && j > 0) ? hz0m + c.ce * (x0m - x00 - y0m + ypm) : T(0);
+  const T hm0 = (ye && i > 0) ? hzm0 + c.ce * (xm0 - xmp - ym0 + y00) : T(0);
+  T e0 = T(0), an_acc = vx0 * x00;
+  an_acc = an_acc + vxm * xm0;
+  // ---- x edge (i, j)
+  T outx, avx1;
+  {
+    const T avt = avx0 + c.cj * (n00 + np0) * x00;
+    T out = x00;
+    if (j == 1 && mb) out = out + b0;
+    if (j == ny - 1 && mt) out = out + t0;
+    if (j == 0 && mb) out = -c.mur * b0;
+    if (j == ny && mt) out = -c.mur * t0;
+    out = out - c.vb * avt;
+    out = out - c.ch * (h00 - h0m);
+    if (c.accum) {
+      const T wl = (i > 0) ? T(0.5) : T(1);                 // node i: this is its right edge
+      const T wr = (i + 1 < nx) ? T(0.5) : T(1);            // node i+1: its left edge
+      out = out + T(2) * ex * (s00 * wl + sp0 * wr);
     }
-    if (i > 0 && i - 1 < nx && j > 0 && j < ny) an_acc = an_acc + f.vx[id - 1] * adj_x(a, md, c.mur, i - 1, j);
-    // ---- y edge (i, j)
-    T outy = T(0), avy1 = T(0);
-    if (ye) {
-      const T phi = c.sphi * c.ckx[i] - c.cphi * c.skx[i];
-      T out, avt;
-      if (i > 0 && i < nx) {
-        const T aEa = adj_y(a, md, c.mur, i, j);
-        avt = avy0 + c.cj * (f.n[id] + f.n[id + p]) * aEa;
-        out = aEa;
-        if (i == 1 && md.m[SIDE_LEFT] == BC_MUR) out = out + a.aEy_in[j * p];
-        if (i == nx - 1 && md.m[SIDE_RIGHT] == BC_MUR) out = out + a.aEy_in[j * p + nx];
-        an_acc = an_acc + f.vy[id] * aEa;
-      } else {
-        const int sd = i == 0 ? SIDE_LEFT : SIDE_RIGHT;
-        avt = avy0;
-        out = md.m[sd] == BC_MUR ? -c.mur * a.aEy_in[id] : T(0);
-      }
-      out = out - c.vb * avt;
-      e0 -= c.vb * avt * phi;
-      T hs = T(0);
-      if (i < nx) hs = hs - h00;
-      if (i > 0) hs = hs + hm0;
-      out = out - c.ch * hs;
-      if (c.accum) {
-        const T ey = f.Ey[id] + c.E0 * phi;
-        const T wb = (j > 0) ? T(0.5) : T(1);
-        const T wt = (j + 1 < ny) ? T(0.5) : T(1);
-        const T g = T(2) * ey * (a.aS2[id] * wb + a.aS2[id + p] * wt);
-        out = out + g;
-        e0 += g * phi;
-      }
-      avy1 = c.va * avt;
-      if (s_l) out = v_l + out;
-      if (s_r) out = v_r + out;
-      outy = out;
+    avx1 = c.va * avt;
+    if (s_b) out = v_b + out;
+    if (s_t) out = v_t + out;
+    outx = out;
+  }
+  // ---- y edge (i, j)
+  an_acc = an_acc + vy0 * y00;
+  an_acc = an_acc + vym * y0m;
+  T outy, avy1;
+  {
+    const T phi = c.sphi * ckx - c.cphi * skx;
+    const T avt = avy0 + c.cj * (n00 + n0p) * y00;
+    T out = y00;
+    if (i == 1 && ml) out = out + l0;
+    if (i == nx - 1 && mr) out = out + r0;
+    if (i == 0 && ml) out = -c.mur * l0;
+    if (i == nx && mr) out = -c.mur * r0;
+    out = out - c.vb * avt;
+    if (ye) e0 -= c.vb * avt * phi;
+    out = out - c.ch * (hm0 - h00);
+    if (c.accum && ye) {
+      const T ey = ey0 + c.E0 * phi;
+      const T wb = (j > 0) ? T(0.5) : T(1);
+      const T wt = (j + 1 < ny) ? T(0.5) : T(1);
+      const T g = T(2) * ey * (s00 * wb + s0p * wt);
+      out = out + g;
+      e0 += g * phi;
     }
-    if (j > 0 && i > 0 && i < nx) an_acc = an_acc + f.vy[id - p] * adj_y(a, md, c.mur, i, j - 1);
-    // ---- stores
-    if (xe && ye) a.aHz_out[id] = h00;
-    a.an[id] = an0 + c.cj * an_acc;
-    if (xe) {
-      a.avx[id] = avx1;
-      if (s_b) ct.side[SIDE_BOTTOM][i] = T(0);
-      if (s_t) ct.side[SIDE_TOP][i] = T(0);
-      if (ct.restr && i >= ct.I0 && i < ct.I1 && j >= ct.jlo && j <= ct.jhi) {
-        const T t = outx / (T)ct.r;
-        T* d = ct.fEx + (size_t)(ct.r * (j - ct.J0)) * ct.fp + ct.r * (i - ct.I0);
-        for (int q = 0; q < ct.r; ++q) d[q] += t;
-        outx = T(0);
-      }
-      a.aEx_out[id] = outx;
+    avy1 = c.va * avt;
+    if (s_l) out = v_l + out;
+    if (s_r) out = v_r + out;
+    outy = out;
+  }
+  // ---- stores
+  if (xe && ye) a.aHz_out[id] = h00;
+  a.an[id] = an0 + c.cj * an_acc;
+  if (xe) {
+    a.avx[id] = avx1;
+    if (s_b) ct.side[SIDE_BOTTOM][i] = T(0);
+    if (s_t) ct.side[SIDE_TOP][i] = T(0);
+    if (ct.restr && i >= ct.I0 && i < ct.I1 && j >= ct.jlo && j <= ct.jhi) {
+      const T t = outx / (T)ct.r;
+      T* d = ct.fEx + (size_t)(ct.r * (j - ct.J0)) * ct.fp + ct.r * (i - ct.I0);
+      for (int q = 0; q < ct.r; ++q) d[q] += t;
+      outx = T(0);
     }
-    if (ye) {
-      a.avy[id] = avy1;
-      if (s_l) ct.side[SIDE_LEFT][j] = T(0);
-      if (s_r) ct.side[SIDE_RIGHT][j] = T(0);
-      if (ct.restr && j >= ct.J0 && j < ct.J1 && i >= ct.ilo && i <= ct.ihi) {
-        const T t = outy / (T)ct.r;
-        T* d = ct.fEy + (size_t)(ct.r * (j - ct.J0)) * ct.fp + ct.r * (i - ct.I0);
-        for (int q = 0; q < ct.r; ++q) d[(size_t)q * ct.fp] += t;
-        outy = T(0);
-      }
-      a.aEy_out[id] = outy;
+    a.aEx_out[id] = outx;
+  }
+  if (ye) {
+    a.avy[id] = avy1;
+    if (s_l) ct.side[SIDE_LEFT][j] = T(0);
+    if (s_r) ct.side[SIDE_RIGHT][j] = T(0);
+    if (ct.restr && j >= ct.J0 && j < ct.J1 && i >= ct.ilo && i <= ct.ihi) {
+      const T t = outy / (T)ct.r;
+      T* d = ct.fEy + (size_t)(ct.r * (j - ct.J0)) * ct.fp + ct.r * (i - ct.I0);
+      for (int q = 0; q < ct.r; ++q) d[(size_t)q * ct.fp] += t;
+      outy = T(0);
     }
+    a.aEy_out[id] = outy;
   }
   return e0;
 }
@@ -332,7 +325,7 @@ __device__ __forceinline__ void ka_part_block(const NodePart<T>& P, int k, doubl
 // beside the fine sub-steps of the same coarse step, which neither read nor
 // write them.
 template <class T>
-__global__ void __launch_bounds__(TX * TY) ka_eh(NodePart<T> P0, NodePart<T> P1, CfbT<T> cb, int nb0, int ncfb,
+__global__ void __launch_bounds__(TX * TY, sizeof(T) == 4 ? 4 : 2) ka_eh(NodePart<T> P0, NodePart<T> P1, CfbT<T> cb, int nb0, int ncfb,
                                                  double* e0acc) {
   const int blk = (int)blockIdx.x;
   if (blk < nb0) {
