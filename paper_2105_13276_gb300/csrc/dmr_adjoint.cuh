@@ -91,11 +91,14 @@ struct CoarseT {
 // selects, and 64 registers hold what is in flight.  (With the loads where the
 // formulas need them, behind the edge tests, the compiler kept 32 registers and
 // a thread made one trip to L2 after the other: 13.9 us per launch cold, of 12
-// blocks as of 580.)  512^2, r = 2, 512 steps recorded and reversed, FP32: 27.8
-// to 23.1 ms; 40 x 32 in FP64, 128 steps: 10.7 to 9.5 ms.
+// blocks as of 580.)  near_mur (the block holds nodes whose edges reach a Mur
+// row's share) is the same for the whole block.  512^2, r = 2, 512 steps recorded
+// and reversed, FP32: 27.8 to 23.1 ms, 21.3 ms with the Mur sides' loads and the
+// fine edges' read-modify-writes out of the other blocks' chains; 40 x 32 in
+// FP64, 128 steps: 10.7 to 9.4 ms.
 template <class T>
 __device__ __forceinline__ T ka_e_node(const AdjM<T>& a, const FwdM<T>& f, const Step<T>& c, const Modes& md,
-                                       const CoarseT<T>& ct, int i, int j) {
+                                       const CoarseT<T>& ct, bool near_mur, int i, int j) {
   const int nx = a.nx, ny = a.ny, p = a.p;
   if (i > nx || j > ny) return T(0);
   const int id = j * p + i;
@@ -135,21 +138,28 @@ __device__ __forceinline__ T ka_e_node(const AdjM<T>& a, const FwdM<T>& f, const
   // column 0 or nx of rows j, j - 1
   const bool mb = md.m[SIDE_BOTTOM] == BC_MUR && j <= 2, mt = md.m[SIDE_TOP] == BC_MUR && j >= ny - 2;
   const bool ml = md.m[SIDE_LEFT] == BC_MUR && i <= 2, mr = md.m[SIDE_RIGHT] == BC_MUR && i >= nx - 2;
-  const T b0 = ld(a.aEx_in + i, mb && xe), bm = ld(a.aEx_in + i - 1, mb && i > 0);
-  const T t0 = ld(a.aEx_in + ny * p + i, mt && xe), tm = ld(a.aEx_in + ny * p + i - 1, mt && i > 0);
-  const T l0 = ld(a.aEy_in + j * p, ml && ye), lm = ld(a.aEy_in + (j - 1) * p, ml && j > 0);
-  const T r0 = ld(a.aEy_in + j * p + nx, mr && ye), rm = ld(a.aEy_in + (j - 1) * p + nx, mr && j > 0);
-  auto mur = [&](T v, bool on, T w) { return on ? v + c.mur * w : v; };
-  x00 = mur(mur(x00, mb && j == 1, b0), mt && j == ny - 1, t0);
-  x0p = mur(mur(x0p, mb && j == 0, b0), mt && j == ny - 2, t0);
-  x0m = mur(mur(x0m, mb && j == 2, b0), mt && j == ny, t0);
-  xm0 = mur(mur(xm0, mb && j == 1, bm), mt && j == ny - 1, tm);
-  xmp = mur(mur(xmp, mb && j == 0, bm), mt && j == ny - 2, tm);
-  y00 = mur(mur(y00, ml && i == 1, l0), mr && i == nx - 1, r0);
-  yp0 = mur(mur(yp0, ml && i == 0, l0), mr && i == nx - 2, r0);
-  ym0 = mur(mur(ym0, ml && i == 2, l0), mr && i == nx, r0);
-  y0m = mur(mur(y0m, ml && i == 1, lm), mr && i == nx - 1, rm);
-  ypm = mur(mur(ypm, ml && i == 0, lm), mr && i == nx - 2, rm);
+  T b0 = T(0), t0 = T(0), l0 = T(0), r0 = T(0);
+  if (near_mur) {   // the same for the whole block
+    b0 = ld(a.aEx_in + i, mb && xe);
+    const T bm = ld(a.aEx_in + i - 1, mb && i > 0);
+    t0 = ld(a.aEx_in + ny * p + i, mt && xe);
+    const T tm = ld(a.aEx_in + ny * p + i - 1, mt && i > 0);
+    l0 = ld(a.aEy_in + j * p, ml && ye);
+    const T lm = ld(a.aEy_in + (j - 1) * p, ml && j > 0);
+    r0 = ld(a.aEy_in + j * p + nx, mr && ye);
+    const T rm = ld(a.aEy_in + (j - 1) * p + nx, mr && j > 0);
+    auto mur = [&](T v, bool on, T w) { return on ? v + c.mur * w : v; };
+    x00 = mur(mur(x00, mb && j == 1, b0), mt && j == ny - 1, t0);
+    x0p = mur(mur(x0p, mb && j == 0, b0), mt && j == ny - 2, t0);
+    x0m = mur(mur(x0m, mb && j == 2, b0), mt && j == ny, t0);
+    xm0 = mur(mur(xm0, mb && j == 1, bm), mt && j == ny - 1, tm);
+    xmp = mur(mur(xmp, mb && j == 0, bm), mt && j == ny - 2, tm);
+    y00 = mur(mur(y00, ml && i == 1, l0), mr && i == nx - 1, r0);
+    yp0 = mur(mur(yp0, ml && i == 0, l0), mr && i == nx - 2, r0);
+    ym0 = mur(mur(ym0, ml && i == 2, l0), mr && i == nx, r0);
+    y0m = mur(mur(y0m, ml && i == 1, lm), mr && i == nx - 1, rm);
+    ypm = mur(mur(ypm, ml && i == 0, lm), mr && i == nx - 2, rm);
+  }
   // ---- adjoint of H^{l-1/2} at the cells (i, j), (i, j - 1), (i - 1, j): that
   // of H^{l+1/2} plus ce curlH^T(aE') over the interior edges
   const T h00 = (xe && ye) ? hz00 + c.ce * (x00 - x0p - y00 + yp0) : T(0);
@@ -206,6 +216,13 @@ __device__ __forceinline__ T ka_e_node(const AdjM<T>& a, const FwdM<T>& f, const
     if (s_r) out = v_r + out;
     outy = out;
   }
+  // ---- a8 transposed: the adjoint of a restricted coarse edge goes to its r
+  // fine edges; the first two of each are loaded before anything is stored
+  const bool gx = ct.restr && xe && i >= ct.I0 && i < ct.I1 && j >= ct.jlo && j <= ct.jhi;
+  const bool gy = ct.restr && ye && j >= ct.J0 && j < ct.J1 && i >= ct.ilo && i <= ct.ihi;
+  T* const dx = ct.fEx + ((ptrdiff_t)(ct.r * (j - ct.J0)) * ct.fp + ct.r * (i - ct.I0));
+  T* const dy = ct.fEy + ((ptrdiff_t)(ct.r * (j - ct.J0)) * ct.fp + ct.r * (i - ct.I0));
+  const T dx0 = ld(dx, gx), dx1 = ld(dx + 1, gx), dy0 = ld(dy, gy), dy1 = ld(dy + ct.fp, gy);
   // ---- stores
   if (xe && ye) a.aHz_out[id] = h00;
   a.an[id] = an0 + c.cj * an_acc;
@@ -213,10 +230,11 @@ __device__ __forceinline__ T ka_e_node(const AdjM<T>& a, const FwdM<T>& f, const
     a.avx[id] = avx1;
     if (s_b) ct.side[SIDE_BOTTOM][i] = T(0);
     if (s_t) ct.side[SIDE_TOP][i] = T(0);
-    if (ct.restr && i >= ct.I0 && i < ct.I1 && j >= ct.jlo && j <= ct.jhi) {
+    if (gx) {
       const T t = outx / (T)ct.r;
-      T* d = ct.fEx + (size_t)(ct.r * (j - ct.J0)) * ct.fp + ct.r * (i - ct.I0);
-      for (int q = 0; q < ct.r; ++q) d[q] += t;
+      dx[0] = dx0 + t;
+      dx[1] = dx1 + t;
+      for (int q = 2; q < ct.r; ++q) dx[q] += t;
       outx = T(0);
     }
     a.aEx_out[id] = outx;
@@ -225,10 +243,11 @@ __device__ __forceinline__ T ka_e_node(const AdjM<T>& a, const FwdM<T>& f, const
     a.avy[id] = avy1;
     if (s_l) ct.side[SIDE_LEFT][j] = T(0);
     if (s_r) ct.side[SIDE_RIGHT][j] = T(0);
-    if (ct.restr && j >= ct.J0 && j < ct.J1 && i >= ct.ilo && i <= ct.ihi) {
+    if (gy) {
       const T t = outy / (T)ct.r;
-      T* d = ct.fEy + (size_t)(ct.r * (j - ct.J0)) * ct.fp + ct.r * (i - ct.I0);
-      for (int q = 0; q < ct.r; ++q) d[(size_t)q * ct.fp] += t;
+      dy[0] = dy0 + t;
+      dy[ct.fp] = dy1 + t;
+      for (int q = 2; q < ct.r; ++q) dy[(size_t)q * ct.fp] += t;
       outy = T(0);
     }
     a.aEy_out[id] = outy;
@@ -313,7 +332,12 @@ template <class T>
 __device__ __forceinline__ void ka_part_block(const NodePart<T>& P, int k, double* e0acc) {
   const int by = P.by0 + k / P.nbx, bx = P.bx0 + k % P.nbx;
   if (bx >= P.sx0 && bx <= P.sx1 && by >= P.sy0 && by <= P.sy1) return;   // whole block
-  const T e0 = ka_e_node(P.a, P.f, P.c, P.md, P.ct, bx * TX + (int)threadIdx.x, by * TY + (int)threadIdx.y);
+  const bool near_mur = (P.md.m[SIDE_LEFT] == BC_MUR && bx * TX <= 2) ||
+                        (P.md.m[SIDE_RIGHT] == BC_MUR && bx * TX + TX - 1 >= P.a.nx - 2) ||
+                        (P.md.m[SIDE_BOTTOM] == BC_MUR && by * TY <= 2) ||
+                        (P.md.m[SIDE_TOP] == BC_MUR && by * TY + TY - 1 >= P.a.ny - 2);
+  const T e0 = ka_e_node(P.a, P.f, P.c, P.md, P.ct, near_mur, bx * TX + (int)threadIdx.x,
+                         by * TY + (int)threadIdx.y);
   const double s = block_sum_d((double)e0);
   if (threadIdx.x == 0 && threadIdx.y == 0 && s != 0.0) atomicAdd(e0acc, s);
 }
