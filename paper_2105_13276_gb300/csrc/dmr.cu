@@ -1406,43 +1406,61 @@ struct Engine final : Base {
     return ck(cudaLaunchKernelEx(&lc, fine_kernel(P.tk), A, G), "fine tile launch");
   }
 
-  // Coarse steps of the next launch, with `left` steps of the period to go
-  // before the caller's end: equal groups of at most K steps (0: strips).
-  // K without the autotuner: 4 for a uniform mesh (1024^2 per step: 11.3 us at
+  // Coarse steps per launch at most (0: strips).  Without the autotuner's
+  // choice: 4 for a uniform mesh (1024^2 per step: 11.3 us at
   // K = 2, 7.0 at 4, 6.9 at 8, 8.1 at 12, where the halos take over), 8 beside a
-  // near region (512^2: 5.3 us per step at K = 4, 4.4 at 8, 4.4 at 12).
-  int multi_steps(int64_t left) {
-    if (!multi_allowed() || left < 2) return 0;
+  // near region (512^2: 5.3 us per step at K = 4, 4.4 at 8, 4.4 at 12), half a
+  // period where the near region is the whole domain.
+  int multi_most() {
+    if (!multi_allowed()) return 0;
     int K = multi_k;
     if (K == 0) {
       const MultiPlan& W = multi_get(2);
       if (!W.ok) return 0;
-      K = W.tk < 0 ? cfg.steps_per_period / 2 : (W.nk < 0 ? 4 : 8);
+      K = W.tk < 0 ? (cfg.steps_per_period + 1) / 2 : (W.nk < 0 ? 4 : 8);
       if (K < 2) K = 2;
     }
-    int64_t g = (left + K - 1) / K;
-    // an even number of launches in a whole period: a captured period then
-    // ends in the buffer parity it starts with
-    if (left == cfg.steps_per_period && (g & 1) && cfg.steps_per_period % 2 == 0) ++g;
-    const int k = (int)((left + g - 1) / g);
-    return multi_get(k).ok ? k : 0;
+    return multi_get(K).ok ? K : 0;
+  }
+  // Coarse steps of the next launch from level mlev on, with `left` steps to
+  // go to the period's end or the caller's (0: strips).  A period is dealt out
+  // once, into an even number of groups that differ by a step at most: it then
+  // ends in the buffer parity it started with, and a captured period can be
+  // replayed.  (Dealt out again after each launch, a period of 60 steps in
+  // groups of 4 took 15 launches, and one whose last steps alone had a plan
+  // mixed both forms; such a period was captured again each time.)  A call that
+  // ends inside a period or starts between groups takes equal groups of its own.
+  int multi_steps(int64_t mlev, int64_t left) {
+    if (left < 2) return 0;
+    const int64_t K = multi_most();
+    if (K == 0) return 0;
+    const int64_t NT = cfg.steps_per_period, q = mlev % NT;
+    if (left == NT - q) {
+      int64_t G = (NT + K - 1) / K;
+      G += G & 1;
+      const int64_t g = (q * G + NT - 1) / NT;     // group g starts at step g NT / G
+      if (g * NT / G == q) {
+        const int k = (int)((g + 1) * NT / G - q);
+        return k < 2 ? 0 : k;
+      }
+    }
+    const int64_t g = (left + K - 1) / K;
+    return (int)((left + g - 1) / g);
   }
 
   // the coarse steps from level mlev on, `left` of them at most to the next
   // stop; *done: steps launched
   int launch_steps(int64_t mlev, int64_t left, int* done) {
-    const int k = multi_steps(left);
+    const int k = multi_steps(mlev, left);
     if (k == 0) {
       *done = 1;
       return launch_coarse_step(mlev);
     }
-    const int fd = fpar ^ (int)(((int64_t)k * cfg.r) & 1);
-    if (int s = go_multi(multi_get(k), mlev, cpar, fpar, fd, pdl_next())) return s;
+    // the fine mesh in place: the near region's cluster holds all of it
+    // between its loads and its stores
+    if (int s = go_multi(multi_get(k), mlev, cpar, fpar, fpar, pdl_next())) return s;
     flip_coarse();
-    if (has_fine) {
-      if (fd != fpar) flip_fine();
-      rvalid = true;
-    }
+    if (has_fine) rvalid = true;
     *done = k;
     return launched("multi-step EM");
   }
@@ -2750,7 +2768,7 @@ struct Engine final : Base {
   // unless a K is more than 1 % faster.
   int autotune_multi(double strip_ms) {
     multi_k = 0;
-    if (!multi_allowed() || multi_steps(cfg.steps_per_period) == 0 || multi_get(2).tk < 0) return DMR_OK;
+    if (!multi_allowed() || multi_most() == 0 || multi_get(2).tk < 0) return DMR_OK;
     const size_t cs2 = L.cplane * sizeof(double);
     const size_t fs2 = has_fine ? (size_t)(F[cur].ny + 1) * (size_t)F[cur].p * sizeof(double) : 0;
     if (int s_ = ck(cudaMemcpyAsync(view, C.S2, cs2, cudaMemcpyDeviceToDevice, st), "keep S2")) return s_;

@@ -1,0 +1,95 @@
+"""Which launches a run's periods are made of: what the rules on sizes choose,
+seen from outside (launch counts and the buffer parities in a saved state)."""
+import numpy as np
+import pytest
+
+pytestmark = pytest.mark.gpu
+
+torch = pytest.importorskip("torch")
+if not torch.cuda.is_available():
+    pytest.skip("needs a CUDA GPU", allow_module_level=True)
+
+from paper_2105_13276_gb300 import dmr as D  # noqa: E402
+from paper_2105_13276_gb300 import workloads as W  # noqa: E402
+
+FIELDS = ("Ex", "Ey", "Hz", "vx", "vy", "n", "S2", "erms")
+
+
+@pytest.fixture(scope="module", autouse=True)
+def _built():
+    from paper_2105_13276_gb300 import build as B
+    B.build()
+    D.load()
+
+
+def _centre(nx, ny, w, h):
+    i, j = (nx - w) // 2, (ny - h) // 2
+    return (i, j, i + w, j + h)
+
+
+def _run(nx, ny, r, rect, NT=64, strips=False, seed=3, **kw):
+    run = D.Run(W.base_cfg(nx=nx, ny=ny, r=r, n_lambda=NT // 2, steps_per_period=NT, precision=1, growth=0, **kw))
+    if r > 1:
+        run.set_patch(rect)
+    if strips:
+        run.set_launch_shape(48)
+    scale = dict(Ex=1e5, Ey=1e5, Hz=3e2, vx=1e4, vy=1e4)
+    for level in range(2 if r > 1 else 1):
+        for k, f in enumerate(scale):
+            run.write(f, level, W.random_fields(run.shape(f, level)[0], seed + 10 * level + k, scale[f]))
+    run.seed_gaussian(1e14, 0.5 * nx * run.dxc, 0.5 * ny * run.dxc, 0.1 * run.lam, 0.1 * run.lam)
+    return run
+
+
+def _equal(a, b, r):
+    for level in range(2 if r > 1 else 1):
+        for f in FIELDS:
+            assert np.array_equal(a.read(f, level), b.read(f, level)), (f, level)
+
+
+def _parities(run):
+    """Buffer parities of the coarse and the fine fields (header of a saved state)."""
+    h = run.save_state()[:40].cpu().numpy().view(np.int32)
+    return int(h[8]), int(h[9])
+
+
+def _launches(run, steps):
+    n = run.launch_count()
+    run.advance(steps)
+    return run.launch_count() - n
+
+
+SHAPES = [(100, 70, 1, 0), (96, 90, 2, 20), (160, 150, 2, 12), (170, 130, 3, 12)]
+
+
+@pytest.mark.parametrize("nx,ny,r,w,NT", [s + (NT,) for s in SHAPES for NT in (20, 36, 60, 63, 64, 100, 120)] +
+                         [(96, 90, 3, 40, 64), (96, 90, 3, 40, 36)])
+def test_a_period_ends_in_the_parity_it_started_with(nx, ny, r, w, NT):
+    """A captured period is replayed only then; each period takes the same
+    launches, fewer than one per step and sub-step, with the same bits."""
+    rect = _centre(nx, ny, w, w) if r > 1 else None
+    a, b = _run(nx, ny, r, rect, NT), _run(nx, ny, r, rect, NT, strips=True)
+    a.set_graphs(True)
+    a.advance(NT)
+    b.advance(NT)
+    par = _parities(a)
+    counts = set()
+    for _ in range(3):
+        counts.add(_launches(a, NT))
+        assert _parities(a) == par
+    assert len(counts) == 1
+    assert counts.pop() < _launches(b, NT)
+    b.advance(2 * NT)
+    _equal(a, b, r)
+
+
+@pytest.mark.parametrize("calls", [(7, 9, 16, 32), (32, 32), (1, 63), (3, 13, 48), (64,), (5, 27, 100, 60)])
+def test_a_period_in_parts(calls):
+    """Calls that stop inside a period and go on between its groups."""
+    for nx, ny, r, w in [(100, 70, 1, 0), (160, 150, 2, 12), (96, 90, 3, 20)]:
+        rect = _centre(nx, ny, w, w) if r > 1 else None
+        a, b = _run(nx, ny, r, rect), _run(nx, ny, r, rect, strips=True)
+        for n in calls:
+            a.advance(n)
+            b.advance(n)
+        _equal(a, b, r)
