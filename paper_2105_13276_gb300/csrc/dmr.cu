@@ -1410,7 +1410,12 @@ struct Engine final : Base {
   // choice: 4 for a uniform mesh (1024^2 per step: 11.3 us at
   // K = 2, 7.0 at 4, 6.9 at 8, 8.1 at 12, where the halos take over), 8 beside a
   // near region (512^2: 5.3 us per step at K = 4, 4.4 at 8, 4.4 at 12), half a
-  // period where the near region is the whole domain.
+  // period where the near region is the whole domain.  A rectangle whose
+  // window does not fit for K takes the largest smaller K that does, where that
+  // beats strips: at r = 2 from 6 steps and 300^2 on (58^2 cells refined, K = 6:
+  // 7.1 us per step against 8.6 at 512^2, 6.8 and 6.9 at 300^2, 6.7 and 6.4 at
+  // 160 x 140; K = 4: 7.8, 7.4, 7.3), at r >= 3 from 3 steps on (r = 3, 43^2
+  // refined, K = 3: 10.4 and 11.3 at 100 x 90, 10.8 and 13.0 at 512^2).
   int multi_most() {
     if (!multi_allowed()) return 0;
     int K = multi_k;
@@ -1420,7 +1425,13 @@ struct Engine final : Base {
       K = W.tk < 0 ? (cfg.steps_per_period + 1) / 2 : (W.nk < 0 ? 4 : 8);
       if (K < 2) K = 2;
     }
-    return multi_get(K).ok ? K : 0;
+    if (multi_get(K).ok) return K;
+    const int least = cfg.r > 2 ? 3 : (double)cfg.nx * cfg.ny >= 90000.0 ? 6 : K;
+    while (K > least) {
+      K = K > 8 ? std::max(8, K / 2) : K - 1;
+      if (multi_get(K).ok) return K;
+    }
+    return 0;
   }
   // Coarse steps of the next launch from level mlev on, with `left` steps to
   // go to the period's end or the caller's (0: strips).  A period is dealt out
@@ -2762,22 +2773,25 @@ struct Engine final : Base {
     return launched("autotune");
   }
 
-  // Coarse steps per launch: K = 4 and 8 (groups of launches as they run, from
-  // the present state into the other buffers; the E^2 sums are kept
-  // aside) against strip_ms per coarse step of the tuned strips.  Strips stay
+  // Coarse steps per launch: K = 4 and 8, or the largest that fits below it
+  // (groups of launches as they run, from the present state into the other
+  // buffers; the E^2 sums are kept aside) against strip_ms per coarse step of the tuned strips.  Strips stay
   // unless a K is more than 1 % faster.
   int autotune_multi(double strip_ms) {
     multi_k = 0;
-    if (!multi_allowed() || multi_most() == 0 || multi_get(2).tk < 0) return DMR_OK;
+    if (!multi_allowed() || !multi_get(2).ok || multi_get(2).tk < 0) return DMR_OK;
     const size_t cs2 = L.cplane * sizeof(double);
     const size_t fs2 = has_fine ? (size_t)(F[cur].ny + 1) * (size_t)F[cur].p * sizeof(double) : 0;
     if (int s_ = ck(cudaMemcpyAsync(view, C.S2, cs2, cudaMemcpyDeviceToDevice, st), "keep S2")) return s_;
     if (has_fine)
       if (int s_ = ck(cudaMemcpyAsync(fS2[cur ^ 1], fS2[cur], fs2, cudaMemcpyDeviceToDevice, st), "keep S2")) return s_;
     double best = strip_ms * 0.99;
-    int best_k = 1;
-    for (int K : {4, 8}) {
+    int best_k = 0;               // 0: none tried, the rule's choice stays
+    int top = 8;
+    while (top > 4 && !multi_get(top).ok) --top;
+    for (int K = 4; K <= top; K = K < top ? top : top + 1) {
       if (K > cfg.steps_per_period || !multi_get(K).ok) continue;
+      if (!best_k) best_k = 1;
       int err = DMR_OK;
       float ms = 0.f;
       const int reps = 2;

@@ -93,3 +93,27 @@ def test_a_period_in_parts(calls):
             a.advance(n)
             b.advance(n)
         _equal(a, b, r)
+
+
+@pytest.mark.parametrize("nx,ny,r,w", [(320, 310, 2, 58), (110, 100, 3, 41), (110, 100, 4, 31), (160, 150, 6, 18)])
+def test_a_rectangle_that_fits_for_fewer_steps_only(nx, ny, r, w):
+    """Too large a window for 8 steps per launch, not for 3 to 7."""
+    rect = _centre(nx, ny, w, w)
+    a, b = _run(nx, ny, r, rect), _run(nx, ny, r, rect, strips=True)
+    assert _launches(a, 64) < 64        # one per coarse step at least otherwise
+    b.advance(64)
+    _equal(a, b, r)
+    a.autotune()
+    a.set_graphs(True)
+    a.advance(128)
+    b.advance(128)
+    _equal(a, b, r)
+
+
+def test_strips_where_a_shorter_group_is_slower():
+    """r = 2 on a small mesh."""
+    nx, ny, w = 160, 140, 58
+    rect = _centre(nx, ny, w, w)
+    a, b = _run(nx, ny, 2, rect), _run(nx, ny, 2, rect, strips=True)
+    assert _launches(a, 64) == _launches(b, 64)
+    _equal(a, b, 2)
