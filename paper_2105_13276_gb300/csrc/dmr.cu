@@ -1456,7 +1456,25 @@ struct Engine final : Base {
       }
     }
     const int64_t g = (left + K - 1) / K;
-    return (int)((left + g - 1) / g);
+    const int k = (int)((left + g - 1) / g);
+    return multi_short(k) ? 0 : k;
+  }
+  // Whether strips are faster than one launch of k <= 4 steps at r = 2: the near
+  // region's loads and stores, shared by few steps, against 7.5 us per coarse
+  // step in strips, more beside a large coarse mesh.  Near nodes (window and
+  // fine mesh) at which the two are equal: about 3000, 8000 and 16000 for 2, 3, 4
+  // (48 x 40, 12^2 refined: 7.7 us against 7.6, 5.8 and 7.1; 96^2, 16^2 refined:
+  // 9.5 and 7.7, 7.2 and 7.2; 120^2: 10.4 and 7.7, 8.2 and 7.3; 512^2, 32^2
+  // refined: 8.7 and 9.5, 7.2 and 8.9; 50^2 refined: 11.0 and 9.6, 8.8 and
+  // 9.1; 200 x 150, 54^2 refined, 4 steps: 7.6 and 7.3).  At r >= 3 the groups
+  // win from 2 steps on.
+  bool multi_short(int k) {
+    if (k > 4 || cfg.r != 2 || !has_fine) return false;
+    const MultiPlan& P = multi_get(k);
+    const double coarse = (double)(cfg.nx + 1) * (cfg.ny + 1);
+    const double near = (double)(P.win[2] - P.win[0] + 1) * (P.win[3] - P.win[1] + 1) +
+                        (double)(F[cur].nx + 1) * (F[cur].ny + 1);
+    return near > (k < 3 ? 3000.0 + coarse / 50.0 : (k < 4 ? 8000.0 : 16000.0) + coarse / 40.0);
   }
 
   // the coarse steps from level mlev on, `left` of them at most to the next

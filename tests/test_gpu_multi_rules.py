@@ -117,3 +117,16 @@ def test_strips_where_a_shorter_group_is_slower():
     a, b = _run(nx, ny, 2, rect), _run(nx, ny, 2, rect, strips=True)
     assert _launches(a, 64) == _launches(b, 64)
     _equal(a, b, 2)
+
+
+@pytest.mark.parametrize("nx,ny,w,strips", [(120, 110, 16, (2, 3)), (70, 64, 16, (2,)), (40, 32, 8, ()),
+                                             (200, 150, 54, (2, 3, 4))])
+def test_calls_of_few_steps(nx, ny, w, strips):
+    """r = 2: two to four steps in one launch only where the near region is small."""
+    rect = _centre(nx, ny, w, w)
+    a, b = _run(nx, ny, 2, rect), _run(nx, ny, 2, rect, strips=True)
+    for k in (2, 3, 4, 2, 5):
+        n, m = _launches(a, k), _launches(b, k)
+        assert m == 2 * k
+        assert n == m if k in strips else n < m, k
+    _equal(a, b, 2)
