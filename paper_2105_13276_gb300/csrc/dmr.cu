@@ -1326,7 +1326,7 @@ struct Engine final : Base {
     int tk = 0, warps = 0, tiles = 0, tw = 0, th = 0, gx = 0, gy = 0, hx = 0;
     size_t smem = 0;
   } fplan;
-  int fine_tiles = 0;      // 0: by rule (r >= 3), 1: no, 2: yes (the autotuner's choice)
+  int fine_tiles = 0;      // 0: by rule (fine_rule), 1: no, 2: yes (the autotuner's choice)
   using FineKernel = void (*)(dmr::MultiArgs<T>, dmr::FineArgs<T>);
   static FineKernel fine_kernel(int tk) {
     if constexpr (sizeof(T) == 4) return tk == 0 ? dmr::k_fine<T, kMC, 2, 1024> : dmr::k_fine<T, kMC, 4, 512>;
@@ -1372,7 +1372,25 @@ struct Engine final : Base {
   }
   bool fine_allowed() const {
     return sizeof(T) == 4 && has_fine && !strips && !timing && !in_batch && !persist_on() && fine_tiles != 1 &&
-           (fine_tiles == 2 || cfg.r >= 3);
+           (fine_tiles == 2 || fine_rule());
+  }
+  // Without the autotuner.  r >= 5: always (1.1 to 1.8 times faster than the
+  // strips from 80 x 40 to 1000^2 fine cells, r = 12 and 16 1.01 to 2.2 times).  r = 3
+  // and 4, captured: the strips' first launch holds the coarse step too, and 3
+  // or 4 launches cost little in a graph, so the tiles win on larger fine meshes
+  // (us per coarse step, strips / tiles, r = 4, 512^2: 160^2 fine 14.7 / 15.7,
+  // 300^2 17.3 / 14.9, 560^2 25.7 / 17.8), and where the coarse step is long (1024^2,
+  // 240^2 fine 21.7 / 21.7) or short (96^2, 160^2 fine 12.3 / 11.7).  Launched one by
+  // one, fewer launches win but at middling coarse sizes (200 x 150, 160^2 fine
+  // 13.7 / 12.9; 512^2, 80^2 fine 15.4 / 16.4) and beside the cheap coarse step of
+  // r = 3 with absorbing layers and the density alone going back (301 x 187,
+  // 180^2 fine 12.9 / 14.1).
+  bool fine_rule() const {
+    if (cfg.r < 3 || cfg.r > 4) return cfg.r > 4;
+    const double fine = (double)(F[cur].nx + 1) * (F[cur].ny + 1), coarse = (double)(cfg.nx + 1) * (cfg.ny + 1);
+    if (!capturing && !(cfg.r == 3 && d.boundary == 1 && d.coupling == 1))
+      return coarse < 200000.0 || coarse >= 500000.0 || fine >= 40000.0;
+    return fine >= 65000.0 || coarse <= 12000.0 || (coarse >= 500000.0 && (cfg.r == 3 || fine >= 28000.0));
   }
   // sub-steps 1 .. r of coarse step mlev: fine parity fp to fp ^ 1, coarse
   // levels n, n + 1 in parities cp, cp ^ 1

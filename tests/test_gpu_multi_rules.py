@@ -130,3 +130,22 @@ def test_calls_of_few_steps(nx, ny, w, strips):
         assert m == 2 * k
         assert n == m if k in strips else n < m, k
     _equal(a, b, 2)
+
+
+@pytest.mark.parametrize("nx,ny,r,w,h,captured,direct", [
+    (200, 150, 4, 40, 40, 4, 2), (200, 150, 4, 80, 60, 2, 2), (200, 150, 3, 50, 50, 3, 2), (200, 150, 2, 70, 60, 2, 2),
+    (512, 400, 4, 40, 40, 4, 4), (512, 400, 4, 60, 50, 4, 2), (200, 150, 5, 30, 30, 2, 2), (100, 96, 4, 40, 36, 2, 2)])
+def test_fine_sub_steps_of_a_small_fine_mesh(nx, ny, r, w, h, captured, direct):
+    """Launches per coarse step of a rectangle too large for the near region:
+    r strips, or the coarse step's and one of fine tiles."""
+    NT, rect = 64, _centre(nx, ny, w, h)
+    a, b = _run(nx, ny, r, rect), _run(nx, ny, r, rect, strips=True)
+    assert _launches(a, 8) == 8 * direct
+    a.advance(NT - 8)
+    a.set_graphs(True)
+    a.advance(NT)
+    b.advance(2 * NT)
+    _equal(a, b, r)
+    end = _launches(b, NT) - r * NT      # the period end's launches
+    assert _launches(a, NT) == captured * NT + end
+    _equal(a, b, r)
