@@ -2801,19 +2801,24 @@ struct Engine final : Base {
         return e_;
       const double per = (double)ms / (kTrialLaunches / 2);
       fine_tiles = per < 0.99 * strip_ms ? 2 : 1;
-      strip_ms = std::min(strip_ms, per);
     }
-    if (int s_ = autotune_multi(strip_ms)) return s_;
+    if (int s_ = autotune_multi()) return s_;
     drop_graph();
     if (wps_out) *wps_out = best_w;
     return launched("autotune");
   }
 
-  // Coarse steps per launch: K = 4 and 8, or the largest that fits below it
-  // (groups of launches as they run, from the present state into the other
-  // buffers; the E^2 sums are kept aside) against strip_ms per coarse step of the tuned strips.  Strips stay
-  // unless a K is more than 1 % faster.
-  int autotune_multi(double strip_ms) {
+  // Coarse steps per launch: K = 4 and 8, or the largest that fits below it,
+  // against one launch per step in the tuned form.  All take about
+  // kTuneSteps coarse steps of a period's middle (every step adds its E^2
+  // sample; a trial at the period boundary, where strips add none, kept them at
+  // r = 4 with 31^2 of 110 x 100 cells refined, 11.8 us per step against
+  // 10.3), launched as they run, from the present state into the other buffers;
+  // the E^2 sums are kept aside.  (A replay costs some 6 us beside its steps:
+  // with 16 of them groups of 4, 9.4 us per step in a period, read 9.7.)  One
+  // step per launch stays unless a K is more than 1 % faster.
+  static constexpr int kTuneSteps = 32;
+  int autotune_multi() {
     multi_k = 0;
     if (!multi_allowed() || !multi_get(2).ok || multi_get(2).tk < 0) return DMR_OK;
     const size_t cs2 = L.cplane * sizeof(double);
@@ -2821,25 +2826,52 @@ struct Engine final : Base {
     if (int s_ = ck(cudaMemcpyAsync(view, C.S2, cs2, cudaMemcpyDeviceToDevice, st), "keep S2")) return s_;
     if (has_fine)
       if (int s_ = ck(cudaMemcpyAsync(fS2[cur ^ 1], fS2[cur], fs2, cudaMemcpyDeviceToDevice, st), "keep S2")) return s_;
-    double best = strip_ms * 0.99;
+    const int64_t lev = m + 1;
+    // time of `launch`, in which err may be set; *per: per coarse step of n
+    int err = DMR_OK;
+    auto trial = [&](const std::function<void()>& launch, int n, double* per) -> int {
+      const int64_t l0 = launches;
+      float ms = 0.f;
+      const int s_ = ck(graph_time(st, launch, 1, &ms), "autotune trial (several steps)");
+      launches = l0 + 4 * (launches - l0);
+      *per = (double)ms / n;
+      return s_ ? s_ : err;
+    };
+    std::vector<dmr::EmArgs<T>> A(cfg.r + 1);      // the coarse step, then fine sub-steps 1..r
+    em_args_for(1, lev, cpar, fpar, true, &A[0], has_fine ? &A[1] : nullptr);
+    for (int k = 2; has_fine && k <= cfg.r; ++k) em_args_for(k, lev, cpar, fpar, true, nullptr, &A[k]);
+    double best = 0.0;
+    int s_ = trial([&]() {
+      for (int q = 0; q < kTuneSteps && !err; ++q) {
+        const int n0 = A[0].nblk + A[0].ncfb;
+        counted(has_fine ? (fine_tiles == 2 ? 2 : cfg.r) : 1);
+        if (!has_fine) {
+          go_em(n0, A[0], q > 0);
+        } else if (fine_tiles == 2) {
+          go_em(n0, A[0], q > 0);
+          err = go_fine(fine_plan(), lev, cpar, fpar, true);
+        } else {
+          go_em2(n0 + A[1].nblk + A[1].ncfb, A[0], A[1], q > 0);
+          for (int k = 2; k <= cfg.r; ++k) go_em(A[k].nblk + A[k].ncfb, A[k], true);
+        }
+      }
+    }, kTuneSteps, &best);
+    if (s_) return s_;
+    best *= 0.99;
     int best_k = 0;               // 0: none tried, the rule's choice stays
     int top = 8;
     while (top > 4 && !multi_get(top).ok) --top;
     for (int K = 4; K <= top; K = K < top ? top : top + 1) {
       if (K > cfg.steps_per_period || !multi_get(K).ok) continue;
       if (!best_k) best_k = 1;
-      int err = DMR_OK;
-      float ms = 0.f;
-      const int reps = 2;
-      auto launch = [&]() {
+      const int reps = (kTuneSteps + K - 1) / K;
+      double per = 0.0;
+      last_em = false;
+      s_ = trial([&]() {
         for (int q = 0; q < reps && !err; ++q)
-          err = go_multi(multi_get(K), m, cpar, fpar, fpar ^ 1, q > 0 && pdl_next());
-      };
-      const int64_t l0 = launches;
-      int s_ = ck(graph_time(st, launch, 1, &ms), "autotune trial (several steps)");
-      launches = l0 + 4 * (launches - l0);
-      if (s_ || err) return s_ ? s_ : err;
-      const double per = (double)ms / ((double)reps * K);
+          err = go_multi(multi_get(K), lev, cpar, fpar, fpar ^ 1, q > 0 && pdl_next());
+      }, reps * K, &per);
+      if (s_) return s_;
       if (per < best) { best = per; best_k = K; }
     }
     multi_k = best_k;

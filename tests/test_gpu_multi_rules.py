@@ -149,3 +149,17 @@ def test_fine_sub_steps_of_a_small_fine_mesh(nx, ny, r, w, h, captured, direct):
     end = _launches(b, NT) - r * NT      # the period end's launches
     assert _launches(a, NT) == captured * NT + end
     _equal(a, b, r)
+
+
+def test_the_autotuner_compares_like_with_like():
+    """Groups of 6 or 7 steps, 15 % faster here than the tuned form of one step
+    (timed without its E^2 sample that form was chosen); the run is as before."""
+    nx, ny, r, w = 110, 100, 4, 31
+    rect = _centre(nx, ny, w, w)
+    a, b = _run(nx, ny, r, rect), _run(nx, ny, r, rect, strips=True)
+    a.set_graphs(True)
+    a.autotune()
+    _equal(a, b, r)
+    assert _launches(a, 64) < 64
+    b.advance(64)
+    _equal(a, b, r)
