@@ -285,11 +285,13 @@ int dmr_sync(const dmr_ctx* ctx);
  * higher targets (shorter strips).  In FP32 runs without CPML each
  * combination is also timed with two node columns per lane in sub-steps
  * 2..r (dmr_set_strip_columns); two must be more than 1 % faster to be
- * chosen.  Last, FP32 runs with Mur sides time groups of launches that advance
- * 4 and 8 coarse steps each, and runs without them the coarse step's launch
- * with one launch of all r fine sub-steps; each is taken where it is more than
- * 1 % faster per coarse step.  *warps_per_sm returns the merged launch's choice
- * (dmr_get_launch_shape gives the whole shape). */
+ * chosen.  Last, FP32 runs time the coarse step's launch with one launch of all
+ * r fine sub-steps, and with Mur sides groups of launches that advance 4 and 8
+ * coarse steps each (a smaller number where the rectangle is too large for 8);
+ * each is taken where it is more than 1 % faster per coarse step.  A shape set
+ * before (dmr_set_launch_shape, dmr_set_strip_columns) is replaced.
+ * *warps_per_sm returns the merged launch's choice (dmr_get_launch_shape gives
+ * the strips' whole shape). */
 int dmr_autotune(dmr_ctx* ctx, int32_t* warps_per_sm, double trial_ms[5]);
 
 /* Duration of one EM launch form of the present step (at a period boundary;
@@ -307,11 +309,12 @@ int dmr_autotune(dmr_ctx* ctx, int32_t* warps_per_sm, double trial_ms[5]);
 int dmr_time_launch(dmr_ctx* ctx, int form, int reps, double* ms_per_launch, double* algorithmic_bytes);
 
 /* Set the strip height of all EM launches directly, as a warps-per-SM target
- * in [1, 1024] (e.g. the choice dmr_autotune made on an earlier run of the
- * same size).  Results do not depend on it.  The run then takes one launch per
- * EM step and sub-step; otherwise an FP32 run with Mur sides may advance
- * several coarse steps per launch (same bits), as dmr_autotune or a rule on
- * the sizes finds faster.  DMR_EINVAL otherwise. */
+ * in [1, 1024].  Results do not depend on it.  The run then takes one launch per
+ * EM step and sub-step until dmr_autotune is called; otherwise an FP32 run may
+ * take all fine sub-steps of a coarse step or several coarse steps per launch
+ * (same bits), as dmr_autotune or a rule on the sizes finds faster.  So the
+ * strip height that dmr_autotune returned is not its whole choice: a later run
+ * of the same size calls dmr_autotune itself.  DMR_EINVAL otherwise. */
 int dmr_set_launch_shape(dmr_ctx* ctx, int32_t warps_per_sm);
 
 /* Node columns each lane of the EM strip kernel advances in the fine

@@ -270,7 +270,7 @@ struct Base {
   cudaGraphExec_t gexec = nullptr;
   int g_cpar = 0, g_fpar = 0, g_rvalid = 0;   // state the graph was captured in
   int g_cend = 0, g_fend = 0;                 // buffer parities its launches leave
-  bool strips = false;                 // one launch per EM (sub-)step only (set by an explicit launch shape)
+  bool strips = false;                 // one launch per EM (sub-)step only (an explicit launch shape, until the autotuner runs)
   std::vector<int32_t> replay;
   size_t replay_pos = 0;
   bool has_fine = false;
@@ -2696,6 +2696,7 @@ struct Engine final : Base {
 
   int autotune(int32_t* wps_out, double* trial_ms) override {
     if (m % cfg.steps_per_period != 0) return fail(DMR_ESTATE, "autotune at a period boundary");
+    strips = false;               // the choice replaces a shape set before
     const int cand[5] = {8, 16, 32, 48, 96};
     // node columns per lane of the later fine sub-steps tried: 1, and 2
     // where the run can use them; two must be more than 1 % faster
@@ -3475,7 +3476,10 @@ struct Batch final : BatchBase {
       launches += 4 * 5;
       if (tune_ms[c] < best) { best = tune_ms[c]; best_w = cand[c]; }
     }
-    for (auto* e : runs) e->warps_per_sm = e->warps_per_sm_fine = best_w;
+    for (auto* e : runs) {
+      e->warps_per_sm = e->warps_per_sm_fine = best_w;
+      e->strips = false;
+    }
     tuned_wps = best_w;
     return build_tables();
   }

@@ -239,7 +239,8 @@ class Run:
         self._check(self.lib.dmr_test_stall(self.ctx, int(bool(on)), int(polls)))
 
     def set_launch_shape(self, warps_per_sm):
-        """Strip height of the EM launches as a warps-per-SM target."""
+        """Strip height of the EM launches as a warps-per-SM target; one launch
+        per EM step and sub-step until the next autotune."""
         self._check(self.lib.dmr_set_launch_shape(self.ctx, int(warps_per_sm)))
 
     def set_strip_columns(self, columns_per_lane):

@@ -163,3 +163,16 @@ def test_the_autotuner_compares_like_with_like():
     assert _launches(a, 64) < 64
     b.advance(64)
     _equal(a, b, r)
+
+
+@pytest.mark.parametrize("force", [lambda run: run.set_launch_shape(48), lambda run: run.set_strip_columns(2)])
+def test_the_autotuner_replaces_a_forced_shape(force):
+    nx, ny, r, w = 200, 150, 3, 20
+    rect = _centre(nx, ny, w, w)
+    a, b = _run(nx, ny, r, rect), _run(nx, ny, r, rect, strips=True)
+    force(a)
+    assert _launches(a, 64) == _launches(b, 64)
+    a.autotune()
+    assert _launches(a, 64) < 64
+    b.advance(64)
+    _equal(a, b, r)
