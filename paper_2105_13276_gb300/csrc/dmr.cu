@@ -1857,7 +1857,7 @@ struct Engine final : Base {
     if (user && (es == 4 || es == 8) && (uintptr_t)user % es == 0 && cudaGetDevice(&dev) == cudaSuccess &&
         cudaPointerGetAttributes(&at, user) == cudaSuccess && at.type == cudaMemoryTypeDevice && at.device == dev) {
       const dim3 g((cols + dmr::kCopyX * dmr::kCopyU - 1) / (dmr::kCopyX * dmr::kCopyU),
-                   (rows + dmr::kCopyY - 1) / dmr::kCopyY);
+                   std::min((rows + dmr::kCopyY - 1) / dmr::kCopyY, dmr::kCopyRows));
       const dim3 b(dmr::kCopyX, dmr::kCopyY);
       if (es == 4) dmr::k_copy2d<float><<<g, b, 0, st>>>((float*)dst, dp, (const float*)src, sp, cols, rows);
       else dmr::k_copy2d<double><<<g, b, 0, st>>>((double*)dst, dp, (const double*)src, sp, cols, rows);
