@@ -4,6 +4,7 @@
 #include <cuda_runtime.h>
 
 #include <algorithm>
+#include <array>
 #include <cmath>
 #include <cstdarg>
 #include <cstdio>
@@ -1086,18 +1087,42 @@ struct Engine final : Base {
     if constexpr (sizeof(T) == 4) return {{1, 1024, dmr::k_near<T, 1, 1024>}, {2, 1024, dmr::k_near<T, 2, 1024>}};
     else return {};
   }
+  // What a plan asks of the runtime once per run and not at each growth of the
+  // rectangle: the kernels' shared-memory limits, and the blocks of a tile
+  // kernel on an SM (at most 4 count) per warps and shared memory.  A captured
+  // period with a growth: 512^2, r = 2, 485 to 469 us; 200 x 150, r = 3, 562 to 548.
+  bool multi_ready = false;
+  std::vector<std::array<size_t, 4>> tile_occ;   // kernel, warps, shared memory, blocks
+  void multi_attributes() {
+    if (multi_ready) return;
+    for (const auto& k : tile_kernels())
+      cudaFuncSetAttribute(k.f, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kMaxSmem);
+    for (const auto& k : near_kernels()) {
+      cudaFuncSetAttribute(k.f, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kMaxSmem);
+      cudaFuncSetAttribute(k.f, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+    }
+    for (int q = 0; q < 2 && sizeof(T) == 4; ++q)
+      cudaFuncSetAttribute(fine_kernel(q), cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kMaxSmem);
+    multi_ready = true;
+  }
+  int tile_blocks(int q, int w, size_t smem) {
+    for (const auto& o : tile_occ)
+      if (o[0] == (size_t)q && o[1] == (size_t)w && o[2] == smem) return (int)o[3];
+    int n = 0;
+    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, tile_kernels()[q].f, 32 * w, smem) != cudaSuccess) {
+      cudaGetLastError();
+      return 0;
+    }
+    tile_occ.push_back({(size_t)q, (size_t)w, smem, (size_t)std::min(n, 4)});
+    return std::min(n, 4);
+  }
   // What a launch of `tiles` tiles of H rows costs, w warps each on sms SMs: the
   // rows that the busiest SM steps, times what a row costs where n blocks
   // share it (one's loads and stores overlap another's steps; 1024^2 at K = 4,
   // relative: 2.9 for one block per SM, 2.4, 2.0 and 1.8 for two, three, four).
-  double tile_cost(int q, int w, size_t smem, long long tiles, int H, int sms) const {
-    int per_sm = 0;
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, tile_kernels()[q].f, 32 * w, smem) != cudaSuccess ||
-        per_sm < 1) {
-      cudaGetLastError();
-      return 1e300;
-    }
-    per_sm = std::min(per_sm, 4);
+  double tile_cost(int q, int w, size_t smem, long long tiles, int H, int sms) {
+    const int per_sm = tile_blocks(q, w, smem);
+    if (per_sm < 1) return 1e300;
     const double f[5] = {0.0, 2.9, 2.4, 2.0, 1.8};
     const int n = (int)std::min<long long>(per_sm, (tiles + sms - 1) / sms);
     const long long rounds = (tiles + (long long)sms * n - 1) / ((long long)sms * n);
@@ -1133,12 +1158,7 @@ struct Engine final : Base {
     P.K = K;
     for (int q = 0; q < 4; ++q) P.rect[q] = has_fine ? rect[q] : -1;
     const int r = cfg.r, nx = cfg.nx, ny = cfg.ny;
-    for (const auto& k : tile_kernels())
-      cudaFuncSetAttribute(k.f, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kMaxSmem);
-    for (const auto& k : near_kernels()) {
-      cudaFuncSetAttribute(k.f, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kMaxSmem);
-      cudaFuncSetAttribute(k.f, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
-    }
+    multi_attributes();
     P.zone[0] = P.zone[1] = 1; P.zone[2] = P.zone[3] = 0;
     bool whole = false;           // the near region is the whole domain: no tiles
     if (has_fine) {
@@ -1347,8 +1367,7 @@ struct Engine final : Base {
     P.tw = (W - 2 * P.hx) / g * g;
     if (P.tw > 0 && nx + 1 >= W) {
       P.gx = (nx + 1 + P.tw - 1) / P.tw;
-      for (const auto& k : tile_kernels())
-        cudaFuncSetAttribute(k.f, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kMaxSmem);
+      multi_attributes();
       double best = 1e300;
       const auto kt = tile_kernels();
       for (size_t q = 0; q < kt.size(); ++q)
@@ -1364,8 +1383,6 @@ struct Engine final : Base {
           P.smem = dmr::fine_smem<T, kMC>(w, kt[q].R, r);
         }
       P.ok = P.warps > 0;
-      for (int q = 0; q < 2 && P.ok; ++q)
-        cudaFuncSetAttribute(fine_kernel(q), cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kMaxSmem);
     }
     fplan = P;
     return fplan;
