@@ -1185,9 +1185,10 @@ struct Engine final : Base {
         }
         return P.nk >= 0;
       };
-      const int all = std::max(nx, ny);
-      if ((double)nx * ny <= kWholeCells && fits(all)) whole = true;
-      else if (!fits(2 * K + 1)) return P;
+      const int all = std::max(nx, ny), mw = 2 * K + 1;
+      const bool covered = rect[0] <= mw && rect[1] <= mw && rect[2] + mw >= nx && rect[3] + mw >= ny;
+      if ((double)nx * ny <= kWholeCells && (!in_batch || covered) && fits(all)) whole = true;
+      else if (!fits(mw)) return P;
       const int m = whole ? all : K;
       P.zone[0] = std::max(rect[0] - m, 0); P.zone[1] = std::max(rect[1] - m, 0);
       P.zone[2] = std::min(rect[2] + m, nx); P.zone[3] = std::min(rect[3] + m, ny);
@@ -1225,7 +1226,11 @@ struct Engine final : Base {
   }
   // a domain of at most this many cells is stepped whole by the near region's
   // cluster, half a period per launch (96^2: 3.8 us per coarse step; tiles of
-  // a domain this small would be mostly halo)
+  // a domain this small would be mostly halo).  Not in a batch, unless the
+  // window is the whole domain anyway: whole domains take a cluster's SMs for
+  // themselves, 7 clusters at a time, tiles and small windows share them (us per
+  // step, r = 2, whole and tiled, 10^2 cells refined: 8 runs of 100^2 10.8 and 5.9,
+  // 64 of 140^2 71.6 and 24.9; 50^2 refined, 8 runs of 140^2 13.2 and 13.2)
   static constexpr double kWholeCells = 20000.0;
 
   // the plan for K steps, kept while the rectangle stays
@@ -3221,7 +3226,8 @@ struct Batch final : BatchBase {
   }
 
   // ---- several coarse steps per launch (dmr_multi.cuh): the whole periods of
-  // FP32 runs that all have a near region.  One launch of tiles and one of
+  // FP32 runs that all have a near region, unless they are many small ones
+  // (group_time).  One launch of tiles and one of
   // near regions (a cluster per run) per K steps and kMultiRuns runs, side by
   // side on two streams.  k_em_batch holds 94 registers (its arguments come
   // from shared memory) and streams each step's state: 16 runs of 128^2 to
@@ -3230,6 +3236,7 @@ struct Batch final : BatchBase {
     bool ok = false;
     int K = 0, twarps = 0, nk = 0, nwarps = 0;
     size_t tsmem = 0, nsmem = 0;
+    double tcost = 0.0;    // tile_cost of the tiles
     std::vector<typename Engine<T>::MultiPlan> run;
   };
   MultiBatchPlan multi_plan() {
@@ -3267,7 +3274,7 @@ struct Batch final : BatchBase {
         for (size_t q = 0; q < runs.size(); ++q)
           if (P.run[q].tk >= 0) tiles += (long long)P.run[q].gx * ((runs[q]->cfg.ny + 1 + th - 1) / th);
         const double cost = runs[0]->tile_cost(0, w, dmr::tile_smem<T, Engine<T>::kMC>(w, P.K), tiles, H, runs[0]->num_sms);
-        if (cost < best) { best = cost; P.twarps = w; }
+        if (cost < best) { best = cost; P.twarps = w; P.tcost = tiles ? cost : 0.0; }
       }
       if (P.twarps == 0) return P;
       P.tsmem = dmr::tile_smem<T, Engine<T>::kMC>(P.twarps, P.K);
@@ -3290,8 +3297,30 @@ struct Batch final : BatchBase {
       P.ok = P.nsmem + 2048 <= Engine<T>::kMaxSmem &&
              cudaOccupancyMaxActiveClusters(&n, kn, &lc) == cudaSuccess && n > 0;
       if (!P.ok) cudaGetLastError();
+      else P.ok = group_time(P, n, NR) <= strip_time();
     }
     return P;
+  }
+  // Estimates in us per coarse step that choose between the two forms, fitted to
+  // batches of 1 to 100 equal runs (70^2 to 256^2 cells, 10^2 to 50^2 of them
+  // refined, r = 2, 4, 8; within 10 % rms): the chosen form was within 2 % of the
+  // better one in all.  The near regions take turns, n clusters at a time; a
+  // turn's time follows the rows that a block's warps step, and is longer where
+  // clusters share SMs; the tiles' work comes on top.  us per step, groups and
+  // strips: 24 runs of 100^2, 24^2 refined 19.2 and 22.2, 64 runs 45.8 and 43.7, 100
+  // runs 83.7 and 67.4 (10^2 refined 30.8 and 43.8).
+  double group_time(const MultiBatchPlan& P, int n, int NR) const {
+    const int turns = ((int)runs.size() + n - 1) / n;
+    const double shared = (double)std::min<int>(n, (int)runs.size()) * Engine<T>::kNearBlocks / runs[0]->num_sms;
+    return turns * (1.0 + 0.2 * std::max(0.0, shared - 1.0)) * (17.4 / P.K + r * (0.62 + 0.0172 * P.nwarps * NR)) +
+           0.0153 * P.tcost;
+  }
+  double strip_time() const {
+    double t = 4.7 * r;
+    for (const auto* e : runs)
+      t += 0.073 * r + 22e-6 * (e->cfg.nx + 1) * (e->cfg.ny + 1) +
+           30e-6 * r * (double)(e->F[e->cur].nx + 1) * (e->F[e->cur].ny + 1);
+    return t;
   }
 
   // a whole period's coarse steps from level m0, host parities cp; launches counted in *nl
