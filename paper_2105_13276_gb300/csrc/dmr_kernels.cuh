@@ -144,6 +144,19 @@ __device__ __forceinline__ double add_sample(double s2, T a, T b, T e, T f) {
   return __fma_rn(0.5, to_f64(mad_(a, a, b * b) + mad_(e, e, f * f)), s2);
 }
 
+// The same for the one-column strips, as the edge path takes it.  FP32 strips
+// wait for their loads and not for the FP64 pipe: halving in FP32, the
+// conversion instruction and an add are the shorter chain (us per coarse step,
+// captured strips, add_sample and this: 512^2 r = 2 8.08 and 7.92, r = 4 13.76 and
+// 13.46, 849 x 274 r = 2 9.18 and 9.05; add_sample with the conversion instruction
+// 8.08, 13.84, 9.28).  The bits are add_sample's while the halves are normal
+// numbers (|E| above 1e-19 V/m).
+template <class T>
+__device__ __forceinline__ double strip_sample(double s2, T a, T b, T e, T f) {
+  if constexpr (sizeof(T) == 4) return s2 + (double)(sq_mean(a, b) + sq_mean(e, f));
+  else return add_sample(s2, a, b, e, f);
+}
+
 // Squared total field at node (i, j): mean of the existing Ex^2 edges along x
 // plus mean of the existing Ey^2 edges along y (incident added to Ey).
 template <class T>
@@ -479,7 +492,7 @@ __device__ __forceinline__ void em_strips_interior(const EmArgs<T>& A, int bx, i
     if (own) {
       dHz[id] = hz;
       if (c.accum) {
-        m.S2[id] = add_sample(cur.s2, exl, exc, eyp + inc, eyc + inc);
+        m.S2[id] = strip_sample(cur.s2, exl, exc, eyp + inc, eyc + inc);
       }
       {
         const T v = upd_v(c, vxo, exc);
