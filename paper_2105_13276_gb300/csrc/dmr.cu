@@ -38,9 +38,12 @@ constexpr int kTrialLaunches = 20;   // launches per autotuner trial graph
 // Mean duration (ms) of one of n back-to-back launches made by `launch`,
 // captured in a CUDA graph on st and replayed (best of three timed replays
 // after one untimed): the periods run as graphs too, and direct launches of
-// small kernels would measure the host's launch rate instead.
+// small kernels would measure the host's launch rate instead.  A first timed
+// replay of more than give_up per launch ends the trial: the autotuner's poor
+// candidates, 2 replays instead of 4.
 template <class F>
-cudaError_t graph_time(cudaStream_t st, F&& launch, int n, float* ms_out) {
+cudaError_t graph_time(cudaStream_t st, F&& launch, int n, float* ms_out, double give_up = 1e30,
+                       int* replays = nullptr) {
   cudaGraph_t g = nullptr;
   cudaGraphExec_t ge = nullptr;
   cudaError_t e = cudaStreamBeginCapture(st, cudaStreamCaptureModeThreadLocal);
@@ -54,18 +57,21 @@ cudaError_t graph_time(cudaStream_t st, F&& launch, int n, float* ms_out) {
   e = cudaEventCreate(&a);
   if (e == cudaSuccess) e = cudaEventCreate(&b);
   float best = 1e30f;
-  for (int rep = 0; rep < 4 && e == cudaSuccess; ++rep) {
+  int rep = 0;
+  for (bool go = true; rep < 4 && go && e == cudaSuccess; ++rep) {
     e = cudaEventRecord(a, st);
     if (e == cudaSuccess) e = cudaGraphLaunch(ge, st);
     if (e == cudaSuccess) e = cudaEventRecord(b, st);
     if (e == cudaSuccess) e = cudaEventSynchronize(b);
     float ms = 0.f;
     if (e == cudaSuccess && rep > 0 && cudaEventElapsedTime(&ms, a, b) == cudaSuccess && ms < best) best = ms;
+    go = rep != 1 || best <= give_up * n;
   }
   if (a) cudaEventDestroy(a);
   if (b) cudaEventDestroy(b);
   cudaGraphExecDestroy(ge);
   *ms_out = best / (float)n;
+  if (replays) *replays = rep;
   return e;
 }
 
@@ -2739,8 +2745,9 @@ struct Engine final : Base {
           go_em(Ac.nblk + Ac.ncfb, Ac);
       };
       float ms = 0.f;
-      if (int s_ = ck(graph_time(st, launch, kTrialLaunches, &ms), "autotune trial")) return s_;
-      launches += 4 * kTrialLaunches;
+      int reps = 0;
+      if (int s_ = ck(graph_time(st, launch, kTrialLaunches, &ms, 1.1 * best, &reps), "autotune trial")) return s_;
+      launches += reps * kTrialLaunches;
       if (trial_ms) trial_ms[c] = ms;
       if (ms < best) { best = ms; best_w = cand[c]; }
     }
@@ -2780,8 +2787,9 @@ struct Engine final : Base {
             }
           };
           float ms = 0.f;
-          if (int s_ = ck(graph_time(st, launch, 1, &ms), "autotune trial (coarse step)")) return s_;
-          launches += 4 * (int64_t)(kTrialLaunches / 2) * cfg.r;
+          int reps = 0;
+          if (int s_ = ck(graph_time(st, launch, 1, &ms, 1.1 * best_p, &reps), "autotune trial (coarse step)")) return s_;
+          launches += reps * (int64_t)(kTrialLaunches / 2) * cfg.r;
           // ties (within 1 %) go to the shorter strips, and to one column per
           // lane
           if (ms < best_p * 0.99 ||
@@ -2817,8 +2825,9 @@ struct Engine final : Base {
         }
       };
       float ms = 0.f;
-      int s_ = ck(graph_time(st, launch, 1, &ms), "autotune trial (fine tiles)");
-      launches += 4 * (int64_t)kTrialLaunches;
+      int reps = 0;
+      int s_ = ck(graph_time(st, launch, 1, &ms, 1.1 * strip_ms * (kTrialLaunches / 2), &reps), "autotune trial (fine tiles)");
+      launches += reps * (int64_t)kTrialLaunches;
       if (s_ || err) return s_ ? s_ : err;
       if (int e_ = ck(cudaMemcpyAsync(fS2[cur], fS2[cur ^ 1], s2b, cudaMemcpyDeviceToDevice, st), "autotune: restore S2"))
         return e_;
@@ -2832,15 +2841,17 @@ struct Engine final : Base {
   }
 
   // Coarse steps per launch: K = 4 and 8, or the largest that fits below it,
-  // against one launch per step in the tuned form.  All take about
-  // kTuneSteps coarse steps of a period's middle (every step adds its E^2
+  // against one launch per step in the tuned form.  All take about 32 coarse
+  // steps (8 without a near region) of a period's middle (every step adds its E^2
   // sample; a trial at the period boundary, where strips add none, kept them at
   // r = 4 with 31^2 of 110 x 100 cells refined, 11.8 us per step against
   // 10.3), launched as they run, from the present state into the other buffers;
-  // the E^2 sums are kept aside.  (A replay costs some 6 us beside its steps:
-  // with 16 of them groups of 4, 9.4 us per step in a period, read 9.7.)  One
-  // step per launch stays unless a K is more than 1 % faster.
-  static constexpr int kTuneSteps = 32;
+  // the E^2 sums are kept aside.  (A replay of groups beside a near region costs
+  // some 5 us more than its steps: with 16 of them strips were kept at 55^2 of
+  // 320 x 310 cells refined, 6.8 us per step against 6.4.)  One step per launch stays
+  // unless a K is more than 1 % faster.  dmr_autotune in all, with 32 steps in every
+  // case and no trial given up early, and now: 512^2 r = 2 20.3 and 15.6 ms, uniform
+  // 1024^2 8.1 and 5.9 ms (the strips' trials alone 16.9 and 5.0).
   int autotune_multi() {
     multi_k = 0;
     if (!multi_allowed() || !multi_get(2).ok || multi_get(2).tk < 0) return DMR_OK;
@@ -2850,13 +2861,15 @@ struct Engine final : Base {
     if (has_fine)
       if (int s_ = ck(cudaMemcpyAsync(fS2[cur ^ 1], fS2[cur], fs2, cudaMemcpyDeviceToDevice, st), "keep S2")) return s_;
     const int64_t lev = m + 1;
+    const int steps = has_fine ? 32 : 8;
     // time of `launch`, in which err may be set; *per: per coarse step of n
     int err = DMR_OK;
-    auto trial = [&](const std::function<void()>& launch, int n, double* per) -> int {
+    auto trial = [&](const std::function<void()>& launch, int n, double* per, double give_up) -> int {
       const int64_t l0 = launches;
       float ms = 0.f;
-      const int s_ = ck(graph_time(st, launch, 1, &ms), "autotune trial (several steps)");
-      launches = l0 + 4 * (launches - l0);
+      int reps = 0;
+      const int s_ = ck(graph_time(st, launch, 1, &ms, give_up * n, &reps), "autotune trial (several steps)");
+      launches = l0 + reps * (launches - l0);
       *per = (double)ms / n;
       return s_ ? s_ : err;
     };
@@ -2865,7 +2878,7 @@ struct Engine final : Base {
     for (int k = 2; has_fine && k <= cfg.r; ++k) em_args_for(k, lev, cpar, fpar, true, nullptr, &A[k]);
     double best = 0.0;
     int s_ = trial([&]() {
-      for (int q = 0; q < kTuneSteps && !err; ++q) {
+      for (int q = 0; q < steps && !err; ++q) {
         const int n0 = A[0].nblk + A[0].ncfb;
         counted(has_fine ? (fine_tiles == 2 ? 2 : cfg.r) : 1);
         if (!has_fine) {
@@ -2878,7 +2891,7 @@ struct Engine final : Base {
           for (int k = 2; k <= cfg.r; ++k) go_em(A[k].nblk + A[k].ncfb, A[k], true);
         }
       }
-    }, kTuneSteps, &best);
+    }, steps, &best, 1e30);
     if (s_) return s_;
     best *= 0.99;
     int best_k = 0;               // 0: none tried, the rule's choice stays
@@ -2887,13 +2900,13 @@ struct Engine final : Base {
     for (int K = 4; K <= top; K = K < top ? top : top + 1) {
       if (K > cfg.steps_per_period || !multi_get(K).ok) continue;
       if (!best_k) best_k = 1;
-      const int reps = (kTuneSteps + K - 1) / K;
+      const int reps = (steps + K / 2) / K;
       double per = 0.0;
       last_em = false;
       s_ = trial([&]() {
         for (int q = 0; q < reps && !err; ++q)
           err = go_multi(multi_get(K), lev, cpar, fpar, fpar ^ 1, q > 0 && pdl_next());
-      }, reps * K, &per);
+      }, reps * K, &per, 1.1 * best);
       if (s_) return s_;
       if (per < best) { best = per; best_k = K; }
     }
