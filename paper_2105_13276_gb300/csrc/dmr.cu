@@ -1506,21 +1506,24 @@ struct Engine final : Base {
     return multi_short(k) ? 0 : k;
   }
   // Whether strips are faster than one launch of k <= 4 steps at r = 2: the near
-  // region's loads and stores, shared by few steps, against 7.5 us per coarse
-  // step in strips, more beside a large coarse mesh.  Near nodes (window and
-  // fine mesh) at which the two are equal: about 3000, 8000 and 16000 for 2, 3, 4
-  // (48 x 40, 12^2 refined: 7.7 us against 7.6, 5.8 and 7.1; 96^2, 16^2 refined:
-  // 9.5 and 7.7, 7.2 and 7.2; 120^2: 10.4 and 7.7, 8.2 and 7.3; 512^2, 32^2
-  // refined: 8.7 and 9.5, 7.2 and 8.9; 50^2 refined: 11.0 and 9.6, 8.8 and
-  // 9.1; 200 x 150, 54^2 refined, 4 steps: 7.6 and 7.3).  At r >= 3 the groups
-  // win from 2 steps on.
+  // region's loads and stores, shared by few steps, against 7.7 us per coarse
+  // step in strips, more beside a large coarse mesh.  What counts is the rows
+  // that a block's warps step (a wide rectangle takes more of them than a tall
+  // one).  us per step, groups and strips, for 2, 3 and 4 steps:
+  //   rows                        2            3            4
+  //   14 (8 x 49 of 150^2)        7.8 / 7.7    6.5 / 7.7    5.7 / 7.4
+  //   18 - 23 (49 x 8, 32^2)      8.7 / 7.7    7.2 / 7.6    6.2 / 7.4
+  //   30 (49 x 8 of 70^2)         9.7 / 7.7    7.9 / 7.5    6.7 / 7.3
+  //   58 (50^2 of 150^2)         11.0 / 7.8    9.1 / 7.8    7.8 / 7.5
+  //   58 (50^2 of 512^2)         11.4 / 10.0   9.4 / 9.6    8.1 / 9.5
+  // At r >= 3 the groups win from 2 steps on.
   bool multi_short(int k) {
     if (k > 4 || cfg.r != 2 || !has_fine) return false;
     const MultiPlan& P = multi_get(k);
+    if (P.nk < 0) return false;
     const double coarse = (double)(cfg.nx + 1) * (cfg.ny + 1);
-    const double near = (double)(P.win[2] - P.win[0] + 1) * (P.win[3] - P.win[1] + 1) +
-                        (double)(F[cur].nx + 1) * (F[cur].ny + 1);
-    return near > (k < 3 ? 3000.0 + coarse / 50.0 : (k < 4 ? 8000.0 : 16000.0) + coarse / 40.0);
+    const double line = k < 3 ? std::max(14.0, coarse / 8500.0) : k < 4 ? 29.0 + coarse / 7500.0 : 52.0 + coarse / 13000.0;
+    return P.nwarps * near_kernels()[P.nk].R > line;
   }
 
   // the coarse steps from level mlev on, `left` of them at most to the next

@@ -132,6 +132,19 @@ def test_calls_of_few_steps(nx, ny, w, strips):
     _equal(a, b, 2)
 
 
+@pytest.mark.parametrize("nx,ny,w,h,strips", [
+    (150, 150, 49, 8, True), (400, 100, 49, 8, True), (400, 100, 8, 49, False), (300, 50, 49, 8, True),
+    (150, 150, 32, 32, True), (512, 512, 32, 32, False), (512, 512, 50, 50, True), (973, 51, 16, 16, False)])
+def test_calls_of_two_steps_by_the_rectangles_shape(nx, ny, w, h, strips):
+    """r = 2: the rows that the near region's warps step, not its nodes."""
+    rect = _centre(nx, ny, w, h)
+    a, b = _run(nx, ny, 2, rect), _run(nx, ny, 2, rect, strips=True)
+    for _ in range(3):
+        n, m = _launches(a, 2), _launches(b, 2)
+        assert (n == m) if strips else (n < m)
+    _equal(a, b, 2)
+
+
 @pytest.mark.parametrize("nx,ny,r,w,h,captured,direct", [
     (200, 150, 4, 40, 40, 4, 2), (200, 150, 4, 80, 60, 2, 2), (200, 150, 3, 50, 50, 3, 2), (200, 150, 2, 70, 60, 2, 2),
     (512, 400, 4, 40, 40, 4, 4), (512, 400, 4, 60, 50, 4, 2), (200, 150, 5, 30, 30, 2, 2), (100, 96, 4, 40, 36, 2, 2)])
