@@ -1410,14 +1410,16 @@ struct Engine final : Base {
   // 300^2 17.3 / 14.9, 560^2 25.7 / 17.8), and where the coarse step is long (1024^2,
   // 240^2 fine 21.7 / 21.7) or short (96^2, 160^2 fine 12.3 / 11.7).  Launched one by
   // one, fewer launches win but at middling coarse sizes (200 x 150, 160^2 fine
-  // 13.7 / 12.9; 512^2, 80^2 fine 15.4 / 16.4) and beside the cheap coarse step of
+  // 13.7 / 12.9; 512^2, 80^2 fine 15.4 / 16.4), for small fine meshes of domains too
+  // narrow for the near region (51 x 973, 80^2 fine 13.3 / 14.4, 160 x 96 fine 14.2 /
+  // 13.6; 60 x 2000, 80^2 fine 15.2 / 12.3) and beside the cheap coarse step of
   // r = 3 with absorbing layers and the density alone going back (301 x 187,
   // 180^2 fine 12.9 / 14.1).
   bool fine_rule() const {
     if (cfg.r < 3 || cfg.r > 4) return cfg.r > 4;
     const double fine = (double)(F[cur].nx + 1) * (F[cur].ny + 1), coarse = (double)(cfg.nx + 1) * (cfg.ny + 1);
     if (!capturing && !(cfg.r == 3 && d.boundary == 1 && d.coupling == 1))
-      return coarse < 200000.0 || coarse >= 500000.0 || fine >= 40000.0;
+      return (coarse < 200000.0 && (fine >= 10000.0 || coarse >= 100000.0)) || coarse >= 500000.0 || fine >= 40000.0;
     return fine >= 65000.0 || coarse <= 12000.0 || (coarse >= 500000.0 && (cfg.r == 3 || fine >= 28000.0));
   }
   // sub-steps 1 .. r of coarse step mlev: fine parity fp to fp ^ 1, coarse

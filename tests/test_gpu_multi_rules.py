@@ -164,6 +164,17 @@ def test_fine_sub_steps_of_a_small_fine_mesh(nx, ny, r, w, h, captured, direct):
     _equal(a, b, r)
 
 
+@pytest.mark.parametrize("nx,ny,r,w,h,direct", [(51, 973, 4, 20, 20, 4), (51, 973, 3, 30, 30, 3), (51, 973, 4, 40, 24, 2),
+                                                (60, 2000, 4, 20, 20, 2)])
+def test_fine_sub_steps_in_a_narrow_domain(nx, ny, r, w, h, direct):
+    """Too narrow for the near region, launched one by one."""
+    rect = _centre(nx, ny, w, h)
+    a, b = _run(nx, ny, r, rect), _run(nx, ny, r, rect, strips=True)
+    assert _launches(a, 8) == 8 * direct
+    b.advance(8)
+    _equal(a, b, r)
+
+
 def test_the_autotuner_compares_like_with_like():
     """Groups of 6 or 7 steps, 15 % faster here than the tuned form of one step
     (timed without its E^2 sample that form was chosen); the run is as before."""
