@@ -114,10 +114,6 @@ struct NearArgs {
 // Tiles
 // ---------------------------------------------------------------------------
 template <class T, int C> struct TileVec;
-template <class T> struct TileVec<T, 1> {
-  static __device__ __forceinline__ void ld(const T* q, T* v) { v[0] = q[0]; }
-  static __device__ __forceinline__ void st(T* q, const T* v) { q[0] = v[0]; }
-};
 template <> struct TileVec<float, 2> {
   static __device__ __forceinline__ void ld(const float* q, float* v) {
     const float2 t = *reinterpret_cast<const float2*>(q);
@@ -156,6 +152,7 @@ __device__ __forceinline__ void multi_tile(const MultiArgs<T>& A, const FineArgs
   const MultiMesh<T>& M = A.C;
   const Mesh<T>& m = M.m;
   const Step<T>& c = M.c;
+  static_assert(C == 2, "float2 and double2 accesses");
   constexpr int W = 32 * C;
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, nw = blockDim.x >> 5;
   const int nx = m.nx, ny = m.ny, p = m.p, K = A.K;
@@ -320,10 +317,8 @@ __device__ __forceinline__ void multi_tile(const MultiArgs<T>& A, const FineArgs
       if constexpr (EDGE) {
         // sides left / right: Eq. 5b, or Mur from the neighbouring column's old and new Ey
         const bool cl = FINE && Fp->mode[SIDE_LEFT] == BC_CFB, cr = FINE && Fp->mode[SIDE_RIGHT] == BC_CFB;
-        const T orr = __shfl_down_sync(0xffffffffu, oy_[0], 1), nrr = __shfl_down_sync(0xffffffffu, ey[q][0], 1);
         const T oll = __shfl_up_sync(0xffffffffu, oy_[C - 1], 1), nll = __shfl_up_sync(0xffffffffu, ey[q][C - 1], 1);
-        if (i0 == 0 && !cl)
-          ey[q][0] = C > 1 ? oy_[C - 1] + c.mur * (ey[q][C - 1] - oy_[0]) : orr + c.mur * (nrr - oy_[0]);
+        if (i0 == 0 && !cl) ey[q][0] = oy_[1] + c.mur * (ey[q][1] - oy_[0]);
 #pragma unroll
         for (int k = 0; k < C; ++k)
           if (i0 + k == nx && !cr)
@@ -376,8 +371,7 @@ __device__ __forceinline__ void multi_tile(const MultiArgs<T>& A, const FineArgs
         TileVec<T, C>::st(M.d[2] + id, hz[q]);
         TileVec<T, C>::st(M.d[3] + id, vx[q]);
         TileVec<T, C>::st(M.d[4] + id, vy[q]);
-        if (C == 2) *reinterpret_cast<double2*>(m.S2 + id) = make_double2(s2[q][0], s2[q][C - 1]);
-        else m.S2[id] = s2[q][0];
+        *reinterpret_cast<double2*>(m.S2 + id) = make_double2(s2[q][0], s2[q][1]);
       }
     } else {
 #pragma unroll
@@ -476,8 +470,7 @@ constexpr int kNearPad = 8;              // rows past the own ones that a unit m
 // edge y from the edge x next to it; IT_PUSH: the old and the new value of
 // coarse edge x to place y of blocks z; IT_LINE: the coarse-fine edge y, sample
 // x), Ey or Ex, and whether the block above keeps a copy (of column IT_COL).
-enum { IT_MUR = 0, IT_PUSH = 1, IT_LINE = 2, IT_OP = 3, IT_Y = 4, IT_UP = 8, IT_DEF = 16, IT_FINE = 32, IT_SIDE = 6,
-       IT_COL = 8 };
+enum { IT_MUR = 0, IT_PUSH = 1, IT_LINE = 2, IT_OP = 3, IT_Y = 4, IT_UP = 8, IT_DEF = 16, IT_FINE = 32, IT_COL = 8 };
 // places for items: the coarse-fine edges (at most two rows and two columns of
 // a block's fine nodes), then the other items of both meshes: as many fine ones
 // (Mur sides), the coarse window's sides, the lines
@@ -523,9 +516,6 @@ __device__ __forceinline__ unsigned cluster_at(unsigned at, int rank) {
 }
 __device__ __forceinline__ void cluster_st(unsigned at, float v) {
   asm volatile("st.shared::cluster.f32 [%0], %1;" ::"r"(at), "f"(v) : "memory");
-}
-__device__ __forceinline__ void cluster_st(unsigned at, double v) {
-  asm volatile("st.shared::cluster.f64 [%0], %1;" ::"r"(at), "d"(v) : "memory");
 }
 
 // What a block needs besides its slabs: the coarse-fine lines, (old, new)
