@@ -1126,6 +1126,7 @@ struct Engine final : Base {
   // rows that the busiest SM steps, times what a row costs where n blocks
   // share it (one's loads and stores overlap another's steps; 1024^2 at K = 4,
   // relative: 2.9 for one block per SM, 2.4, 2.0 and 1.8 for two, three, four).
+  // Other K, the fine tiles and batches take the same weights.
   double tile_cost(int q, int w, size_t smem, long long tiles, int H, int sms) {
     const int per_sm = tile_blocks(q, w, smem);
     if (per_sm < 1) return 1e300;
@@ -1455,10 +1456,10 @@ struct Engine final : Base {
   }
 
   // Coarse steps per launch at most (0: strips).  Without the autotuner's
-  // choice: 4 for a uniform mesh (1024^2 per step: 11.3 us at
-  // K = 2, 7.0 at 4, 6.9 at 8, 8.1 at 12, where the halos take over), 8 beside a
-  // near region (512^2: 5.3 us per step at K = 4, 4.4 at 8, 4.4 at 12), half a
-  // period where the near region is the whole domain.  A rectangle whose
+  // choice: 4 for a uniform mesh (1024^2 per step, period end included: 7.8 us at
+  // K = 2, 6.6 at 4, 7.5 at 6 and 8, 8.3 at 12, where the halos take over), 8 beside
+  // a near region (512^2: 7.9 us per step at K = 2, 6.2 at 4, 5.4 at 8 and 12), half
+  // a period where the near region is the whole domain.  A rectangle whose
   // window does not fit for K takes the largest smaller K that does, where that
   // beats strips: at r = 2 from 6 steps and 300^2 on (58^2 cells refined, K = 6:
   // 7.1 us per step against 8.6 at 512^2, 6.8 and 6.9 at 300^2, 6.7 and 6.4 at

@@ -137,8 +137,9 @@ __device__ __forceinline__ double to_f64_any(float v) {
 // s2 + (a^2 + b^2)/2 + (e^2 + f^2)/2, the E^2 sample of a node with two edges
 // each way: the halves are exact, so one factor 1/2 in the sum's fused
 // multiply-add gives the bits of halving each mean first, and costs two
-// multiplies less (an FMA also takes the FP64 pipe 0.52 clocks per lane and SM,
-// an add 0.63): 512^2 in FP64 with a 64^2 patch 31.55 to 30.83 us per coarse step
+// multiplies less (an FMA also takes the FP64 pipe 16 cycles per warp and SM, an
+// add or a multiply 19): 512^2 in FP64 with a 64^2 patch 31.55 to 30.83 us per
+// coarse step
 template <class T>
 __device__ __forceinline__ double add_sample(double s2, T a, T b, T e, T f) {
   return __fma_rn(0.5, to_f64(mad_(a, a, b * b) + mad_(e, e, f * f)), s2);
@@ -1351,7 +1352,7 @@ struct PeMesh {
 };
 // Node rows per thread of the period-end launches on a larger mesh: a thread
 // adds its rows' terms before the block's sum, which costs five FP64 adds per
-// warp and row (16 cycles of the SM's FP64 pipe each); a smaller mesh keeps one
+// warp and row (19 cycles of the SM's FP64 pipe each); a smaller mesh keeps one
 // row per thread, for the blocks.  FP32, all steps of a period with its end:
 // uniform 1024^2 861 to 840 us, 2048 x 1024 with a quarter refined r = 2 4.24 to
 // 4.12 ms, r = 4 14.02 to 13.72 ms, a batch of 16 runs 8.90 to 8.47 ms.

@@ -11,17 +11,21 @@
 //    writes level n + K into the other buffer parity, as the one-step launches
 //    do.  Two node columns per lane (float2 loads), x neighbours by shuffle,
 //    the rows next to another warp's through shared memory, one block barrier
-//    per step.  Bound by instruction issue and, for the FP64 E^2 sums, by the
-//    FP64 pipe (16 cycles per warp and SM for an add; a conversion would take as
-//    many, see to_f64).  1024^2: 11.4 us per step with one launch each, 6.1 us
-//    with K = 4 (with one block per SM 7.0 us, and 9.1 us with the conversion
-//    instruction); 512^2: 1.8 us of tiles per step at K = 8.
+//    per step.  Issue slots are 58 % used (2 blocks of 15 warps per SM), the FP64
+//    pipe 35 % (the E^2 sums: 16 cycles per warp and SM for a fused multiply-add,
+//    19 for an add, 16 for a conversion, hence to_f64); the rest waits for a tile's
+//    loads, shuffles and the step's barrier.  1024^2 with its period end: 11.4 us
+//    per step with one launch each, 6.6 us with K = 4 (with one block of 32 warps
+//    per SM 8.5 us, with the conversion instruction 8.2 us); 512^2: 1.7 us of tiles
+//    per step at K = 8.
 //
 //  * Fine tiles (k_fine).  The r sub-steps of a larger fine mesh in one launch of
 //    such tiles after the coarse step's launch; the coarse-fine sides blend the
 //    coarse lines of both levels, the last sub-step writes the fine->coarse
 //    means.  2048 x 1024, a quarter of it refined: 392 us per coarse step at
-//    r = 4 with one launch per sub-step, 211 us here; r = 2: 78 to 62 us.
+//    r = 4 with one launch per sub-step, 211 us here; r = 2: 78 to 62 us.  Issue
+//    slots 67 % used on 1200^2 fine cells (blocks of 10 warps), 46 % on 800^2 (one
+//    block of 26 warps per SM, 1.9 waves).
 //
 //  * The near region (k_near).  The fine rectangle with its r sub-steps per
 //    coarse step and the coarse nodes up to 2K + 1 around it live in one
@@ -31,11 +35,12 @@
 //    with one cluster barrier (0.3 us) per sub-step.  It stores the coarse
 //    nodes up to K around the rectangle (what the tiles, which know nothing of
 //    the fine mesh, get wrong) and the fine mesh, and runs beside the tiles on a
-//    stream of its own.  Bound by latency: 3.7 us per coarse step at r = 2 with
-//    a 64^2 patch, where the one-step launches take 4.5 + 2.9 us.
+//    stream of its own.  Bound by latency (a warp is at barriers 44 % of its
+//    time, waiting for instructions 12 %; a fourth of the issue slots used): 3.7 us per coarse step at r = 2 with a 64^2 patch, where the
+//    one-step launches take 4.5 + 2.9 us.
 //
 // 512^2 with a 64^2 patch: 8.2 us per coarse step with one launch per step and
-// sub-step, 4.4 us here (K = 8); 96^2 whole in the cluster: 6.0 to 3.7 us.
+// sub-step, 4.4 us here (K = 8); 96^2 whole in the cluster: 6.0 to 3.4 us.
 //
 // Every element goes through the helpers of dmr_kernels.cuh in the order of
 // the one-step launches, so both give the same bits.
