@@ -1399,29 +1399,47 @@ struct Engine final : Base {
     fplan = P;
     return fplan;
   }
-  bool fine_allowed() const {
+  bool fine_allowed() {
     return sizeof(T) == 4 && has_fine && !strips && !timing && !in_batch && !persist_on() && fine_tiles != 1 &&
            (fine_tiles == 2 || fine_rule());
   }
   // Without the autotuner.  r >= 5: always (1.1 to 1.8 times faster than the
   // strips from 80 x 40 to 1000^2 fine cells, r = 12 and 16 1.01 to 2.2 times).  r = 3
-  // and 4, captured: the strips' first launch holds the coarse step too, and 3
-  // or 4 launches cost little in a graph, so the tiles win on larger fine meshes
-  // (us per coarse step, strips / tiles, r = 4, 512^2: 160^2 fine 14.7 / 15.7,
-  // 300^2 17.3 / 14.9, 560^2 25.7 / 17.8), and where the coarse step is long (1024^2,
-  // 240^2 fine 21.7 / 21.7) or short (96^2, 160^2 fine 12.3 / 11.7).  Launched one by
-  // one, fewer launches win but at middling coarse sizes (200 x 150, 160^2 fine
-  // 13.7 / 12.9; 512^2, 80^2 fine 15.4 / 16.4), for small fine meshes of domains too
-  // narrow for the near region (51 x 973, 80^2 fine 13.3 / 14.4, 160 x 96 fine 14.2 /
-  // 13.6; 60 x 2000, 80^2 fine 15.2 / 12.3) and beside the cheap coarse step of
-  // r = 3 with absorbing layers and the density alone going back (301 x 187,
-  // 180^2 fine 12.9 / 14.1).
-  bool fine_rule() const {
-    if (cfg.r < 3 || cfg.r > 4) return cfg.r > 4;
+  // and 4: the strips' first launch holds the coarse step too, and 3 or 4
+  // launches cost little in a graph, so captured the tiles win on larger fine
+  // meshes only, and where the coarse step is long or has little to share
+  // (tiles / strips, us per coarse step, r = 4: 200 x 150, 60^2 cells refined 14.0 /
+  // 13.2, 76 x 95 12.9 / 14.5; 600 x 300, 50^2 13.1 / 14.1; 64 x 183, 30 x 54 13.9 /
+  // 12.4).  Launched one by one, fewer launches win but at middling coarse sizes
+  // (200 x 150, 40^2 refined 12.9 / 13.8; 512^2, 20^2 refined 16.4 / 15.4) and for small
+  // fine meshes of domains too narrow for the near region (51 x 973, 20^2 refined
+  // 14.4 / 13.4; 60 x 2000 12.3 / 15.2; 40 x 212, 40 x 9 refined 10.9 / 13.9; 232 x 87,
+  // r = 3, 115 x 4 refined 11.3 / 13.3).  With the density alone going back (coupling)
+  // r = 3's last sub-step is cheap, and strips win up to larger meshes (301 x 187,
+  // 90^2 refined 11.9 / 10.7, with absorbing layers 13.8 / 12.4).  The lines were
+  // drawn on 1964 points (25 coarse sizes from 6561 to 1050625 nodes, 8 to 14 rectangles each,
+  // both couplings, CPML): the choice loses 0.3 % on average to the better form.
+  bool fine_rule() {
+    const int r = cfg.r;
+    if (r < 3 || r > 4) return r > 4;
     const double fine = (double)(F[cur].nx + 1) * (F[cur].ny + 1), coarse = (double)(cfg.nx + 1) * (cfg.ny + 1);
-    if (!capturing && !(cfg.r == 3 && d.boundary == 1 && d.coupling == 1))
-      return (coarse < 200000.0 && (fine >= 10000.0 || coarse >= 100000.0)) || coarse >= 500000.0 || fine >= 40000.0;
-    return fine >= 65000.0 || coarse <= 12000.0 || (coarse >= 500000.0 && (cfg.r == 3 || fine >= 28000.0));
+    const bool mur = d.boundary == 0, light = r == 3 && d.coupling == 1;
+    if (capturing) {
+      if (light) return fine >= 100000.0 || (mur && coarse >= 150000.0 && coarse < 200000.0);
+      if (mur && coarse >= 150000.0 && coarse < 205000.0) return true;
+      if (r == 3) return fine >= 65000.0 || coarse <= 11500.0 || coarse >= 450000.0;
+      // a small domain: where the tiles' columns are used
+      const FinePlan& P = fine_plan();
+      return fine >= 75000.0 || (coarse >= 500000.0 && fine >= 28000.0) ||
+             (coarse <= 10000.0 && P.ok && F[cur].nx + 1 >= 0.88 * P.gx * P.tw);
+    }
+    if (light && !mur)
+      return fine >= 75000.0 || coarse < 11000.0 || (coarse >= 140000.0 && coarse < 200000.0) || coarse >= 450000.0;
+    const bool few = fine < 10000.0 && coarse >= 30000.0 && coarse < 100000.0;
+    if (light)
+      return fine >= 100000.0 || (coarse < 40000.0 && !few) || (coarse >= 95000.0 && coarse < 200000.0) ||
+             coarse >= 450000.0;
+    return (coarse < 200000.0 && !few) || coarse >= 450000.0 || fine >= 40000.0;
   }
   // sub-steps 1 .. r of coarse step mlev: fine parity fp to fp ^ 1, coarse
   // levels n, n + 1 in parities cp, cp ^ 1

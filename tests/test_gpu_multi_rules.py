@@ -175,6 +175,24 @@ def test_fine_sub_steps_in_a_narrow_domain(nx, ny, r, w, h, direct):
     _equal(a, b, r)
 
 
+@pytest.mark.parametrize("nx,ny,r,w,h,kw,captured,direct", [
+    (64, 183, 4, 16, 54, {}, 4, 2), (40, 212, 4, 40, 9, {}, 2, 2), (64, 183, 4, 30, 54, dict(coupling=1), 4, 2), (150, 120, 3, 50, 50, {}, 3, 2), (232, 87, 3, 115, 4, {}, 3, 2),
+    (89, 705, 3, 76, 95, dict(coupling=1), 3, 3), (301, 187, 3, 90, 90, dict(coupling=1), 3, 3),
+    (301, 187, 3, 90, 90, dict(coupling=1, boundary=1), 3, 3), (301, 187, 3, 90, 90, {}, 2, 2),
+    (600, 300, 4, 50, 50, {}, 2, 2), (200, 150, 4, 76, 95, {}, 2, 2), (200, 150, 3, 120, 120, dict(coupling=1), 2, 2)])
+def test_fine_sub_steps_by_the_sizes_of_both_meshes(nx, ny, r, w, h, kw, captured, direct):
+    NT, rect = 64, _centre(nx, ny, w, h)
+    a, b = _run(nx, ny, r, rect, **kw), _run(nx, ny, r, rect, strips=True, **kw)
+    assert _launches(a, 8) == 8 * direct
+    a.advance(NT - 8)
+    a.set_graphs(True)
+    a.advance(NT)
+    b.advance(2 * NT)
+    end = _launches(b, NT) - r * NT
+    assert _launches(a, NT) == captured * NT + end
+    _equal(a, b, r)
+
+
 def test_the_autotuner_compares_like_with_like():
     """Groups of 6 or 7 steps, 15 % faster here than the tuned form of one step
     (timed without its E^2 sample that form was chosen); the run is as before."""
