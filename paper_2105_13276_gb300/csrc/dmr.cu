@@ -1908,12 +1908,16 @@ struct Engine final : Base {
     int dev = -1;
     if (user && (es == 4 || es == 8) && (uintptr_t)user % es == 0 && cudaGetDevice(&dev) == cudaSuccess &&
         cudaPointerGetAttributes(&at, user) == cudaSuccess && at.type == cudaMemoryTypeDevice && at.device == dev) {
-      const dim3 g((cols + dmr::kCopyX * dmr::kCopyU - 1) / (dmr::kCopyX * dmr::kCopyU),
-                   std::min((rows + dmr::kCopyY - 1) / dmr::kCopyY, dmr::kCopyRows));
       const dim3 b(dmr::kCopyX, dmr::kCopyY);
-      if (es == 4) dmr::k_copy2d<float><<<g, b, 0, st>>>((float*)dst, dp, (const float*)src, sp, cols, rows);
-      else dmr::k_copy2d<double><<<g, b, 0, st>>>((double*)dst, dp, (const double*)src, sp, cols, rows);
-      counted(1);
+      for (int j = 0; j < rows; j += dmr::kCopyRows) {
+        const int n = std::min(rows - j, dmr::kCopyRows);
+        const dim3 g((cols + dmr::kCopyX * dmr::kCopyU - 1) / (dmr::kCopyX * dmr::kCopyU),
+                     (n + dmr::kCopyY - 1) / dmr::kCopyY);
+        const size_t to = (size_t)j * dp, from = (size_t)j * sp;
+        if (es == 4) dmr::k_copy2d<float><<<g, b, 0, st>>>((float*)dst + to, dp, (const float*)src + from, sp, cols, n);
+        else dmr::k_copy2d<double><<<g, b, 0, st>>>((double*)dst + to, dp, (const double*)src + from, sp, cols, n);
+        counted(1);
+      }
       return launched("field copy");
     }
     cudaGetLastError();

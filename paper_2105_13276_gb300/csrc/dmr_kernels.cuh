@@ -1779,24 +1779,25 @@ __global__ void k_erms_view(Mesh<T> m, Step<T> c, double q, T* out) {
 // of columns), so the accesses are single elements, 128 bytes per warp.  Six
 // fields of both meshes of a 2048 x 1024 run at r = 4 (252 MB): 129 us, with
 // cudaMemcpy2DAsync 304 us; of a 1024 x 1024 mesh 25 against 50 us; at 512 x 512
-// and below the call costs what it did.  More rows than kCopyRows blocks hold
-// (a grid's limit in y) are taken in strides of the grid.
-constexpr int kCopyX = 128, kCopyY = 4, kCopyU = 4, kCopyRows = 65535;
+// and below the call costs what it did.  A launch takes at most kCopyRows rows
+// (a grid's limit in y).  (With the rows in strides of the grid instead, a loop
+// around the kernel's one round of loads, a 10 x 3000 field took 3.9 us, now 3.4.)
+constexpr int kCopyX = 128, kCopyY = 4, kCopyU = 4, kCopyRows = 65535 * kCopyY;
 template <class E>
 __global__ void __launch_bounds__(kCopyX* kCopyY) k_copy2d(E* __restrict__ dst, int dp, const E* __restrict__ src, int sp,
                                                             int cols, int rows) {
   const int i = blockIdx.x * (kCopyX * kCopyU) + threadIdx.x;
-  for (int j = blockIdx.y * kCopyY + threadIdx.y; j < rows; j += gridDim.y * kCopyY) {
-    const E* s = src + (size_t)j * sp;
-    E* d = dst + (size_t)j * dp;
-    E v[kCopyU];
+  const int j = blockIdx.y * kCopyY + threadIdx.y;
+  if (j >= rows) return;
+  const E* s = src + (size_t)j * sp;
+  E* d = dst + (size_t)j * dp;
+  E v[kCopyU];
 #pragma unroll
-    for (int u = 0; u < kCopyU; ++u)
-      if (i + u * kCopyX < cols) v[u] = s[i + u * kCopyX];
+  for (int u = 0; u < kCopyU; ++u)
+    if (i + u * kCopyX < cols) v[u] = s[i + u * kCopyX];
 #pragma unroll
-    for (int u = 0; u < kCopyU; ++u)
-      if (i + u * kCopyX < cols) d[i + u * kCopyX] = v[u];
-  }
+  for (int u = 0; u < kCopyU; ++u)
+    if (i + u * kCopyX < cols) d[i + u * kCopyX] = v[u];
 }
 
 }  // namespace dmr
